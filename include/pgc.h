@@ -226,7 +226,9 @@ const char *pgc_strerror(int32_t code);
  * least squares), "tc_fused" (softmax on the tensor cores, residual in the
  * logits GEMM), "tc" (tensor cores, separate residual kernel),
  * "softmax_rows" (few classes, whole rows per CTA pair), "softmax_cluster" (few
- * classes, 8-CTA clusters), "softmax_cc" (CUDA cores); "" for NULL. */
+ * classes, 8-CTA clusters), "softmax_cc" (single precision: up to 128 classes
+ * on the tensor cores with operands in three bf16 parts, else CUDA cores);
+ * "" for NULL. */
 const char *pgc_gradient_path(const pgc_ctx *ctx);
 
 /* pgc_last_cuda_error — name of the CUDA runtime error behind the most
@@ -316,8 +318,8 @@ int64_t pgc_step_count(const pgc_ctx *ctx);
 /* Kernel groups of one step, in launch order, as counted and timed below.
  * Paths without a group leave it empty (zero time, zero launches). */
 #define PGC_KGRAD   0   /* gradient: streaming row kernel, few-class softmax
-                           kernel, tensor-core logits GEMM, or the CUDA-core
-                           softmax kernels                                     */
+                           kernel, tensor-core logits GEMM, or the single-
+                           precision softmax kernels                                    */
 #define PGC_KRESID  1   /* tensor-core softmax: residual R = softmax(Z) - Y    */
 #define PGC_KGRADB  2   /* tensor-core softmax: gradient GEMM R^T X            */
 #define PGC_KCOMMIT 3   /* gradient-store commit                               */

@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
       }
       float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       w = f4fma(-a.lr, g, w);
-      store_outputs(a, p, g, w);
+      store_outputs_any(a, p, g, w);
     }
     return;
   }
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
     const float4 g = f4fma(pl.B, V, D);
     float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
-    store_outputs(a, p, g, w);
+    store_outputs_any(a, p, g, w);
   }
 }
 

@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(256) gc_decode_kernel(DecodeArgs a, const floa
     }
     float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
-    store_outputs(a, p, g, w);
+    store_outputs_any(a, p, g, w);
   }
 }
 

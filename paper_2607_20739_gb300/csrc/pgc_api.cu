@@ -64,6 +64,10 @@ struct Phase {
   int32_t* d_sk_tiles = nullptr;
   std::vector<int32_t> sk_cuts;   // whole-row variant: tile range of each CTA pair
   int32_t* d_sk_cuts = nullptr;
+  // single-precision softmax on the tensor cores: logits and gradient units
+  std::vector<SplitUnit> sl_units, sg_units;
+  SplitUnit *d_sl_units = nullptr, *d_sg_units = nullptr;
+  int sg_items = 0;               // partials of the gradient units (0: straight into the stores)
   // device copies
   WorkItem* d_items = nullptr;
   int32_t* d_e_item0 = nullptr;
@@ -153,6 +157,14 @@ struct pgc_ctx {
   int tcg_pairs = 0;         // co-resident CTA pairs of the gradient contraction
   alignas(64) unsigned char tmXq[128];   // X as the fused kernel's A part (box 64 x 128/NT)
   alignas(64) unsigned char tmRst[128];  // Rb as the fused kernel's output (box 64 x 32)
+  bool split = false;        // softmax in single precision on the tensor cores
+  int sp_nc = 0;             // its clusters of two CTAs
+  int sp_Kp = 0, sp_C3 = 0;  // classes padded to 16, columns of R
+  int sp_chunk = 0;          // K blocks per accumulator
+  uint16_t* R3 = nullptr;    // residual parts [R rows][C3]
+  void* tmX = nullptr;       // device tensor maps of X: [n] logits, [n] gradient
+  alignas(64) unsigned char tmW3[128];   // W parts [3 Kp][ld]
+  alignas(64) unsigned char tmR3[128];   // R parts
   // GC-CR coding: the naive PGC-CR mode and GC with cyclic repetition (§V-A)
   bool gc_weighted = false;    // decode with GC-CR's weights instead of PGC's slot totals
   bool gc_ready = false;       // encoding coefficients set (pgc_set_gc_encoding)
@@ -206,6 +218,54 @@ int read_status(pgc_ctx* ctx) {
   if (h & kErrSingular) { ctx->broken = true; return PGC_ESINGULAR; }
   if (h) { ctx->broken = true; return PGC_ECUDA; }
   return PGC_OK;
+}
+
+// Units of the single-precision tensor-core softmax kernels.  Logits: 256
+// rows of a partition.  Gradient: 256 features of a run of L rows of a
+// partition; L is the multiple of 64 that minimises the rounds over the
+// clusters times a unit's length (its K blocks plus about six for filling the
+// pipeline and writing out), plus the commit of the partials (a launch, and
+// writing and reading them at about 5 TB/s, in blocks of about 0.3 us) that
+// more than one unit per partition and feature tile costs.
+void build_split_units(pgc_ctx* ctx, Phase& ph) {
+  const int nE = (int)ph.parts.size();
+  const int64_t SP = (ctx->ld + kSplitFeatures - 1) / kSplitFeatures, nc = ctx->sp_nc;
+  int64_t z = 0;
+  std::vector<int32_t> z0(nE);
+  for (int e = 0; e < nE; ++e) {
+    const int64_t m = ph.e_rows[e];
+    z0[e] = (int32_t)z;
+    for (int64_t r = 0; r < m; r += kSplitRows)
+      ph.sl_units.push_back({e, ph.parts[e], (int32_t)ph.e_row0[e], (int32_t)r, (int32_t)m, z0[e], 0, 0});
+    z += (m + 127) / 128 * 128;
+  }
+  ph.zpad_total = z;
+  int64_t best_L = (ph.max_rows + 63) / 64 * 64;
+  double best = 0.0;
+  for (int64_t q = 1; q <= 64; ++q) {
+    const int64_t L = ((ph.max_rows + q - 1) / q + 63) / 64 * 64;
+    if (q > 1 && L < 256) break;
+    int64_t items = 0;
+    for (int e = 0; e < nE; ++e) items += (ph.e_rows[e] + L - 1) / L;
+    const double rounds = (double)((items * SP + nc - 1) / nc);
+    const double commit = items > nE ? 10.0 + (double)items * (double)ctx->P * 8.0 / 5e12 / 0.3e-6 : 0.0;
+    const double cost = rounds * ((double)L / 64.0 + 6.0) + commit;
+    if (q == 1 || cost < best) { best = cost; best_L = L; }
+  }
+  int item = 0;
+  ph.e_item0.push_back(0);
+  for (int e = 0; e < nE; ++e) {
+    for (int64_t r = 0; r < ph.e_rows[e]; r += best_L, ++item)
+      for (int64_t sp = 0; sp < SP; ++sp)
+        ph.sg_units.push_back({e, ph.parts[e], (int32_t)sp, (int32_t)r, (int32_t)std::min(best_L, ph.e_rows[e] - r),
+                               z0[e], item, 0});
+    ph.e_item0.push_back(item);
+  }
+  ph.sg_items = item;
+  if (item == nE) {   // one unit per partition and feature tile: no partials
+    ph.sg_items = 0;
+    for (auto& u : ph.sg_units) u.item = -1;
+  }
 }
 
 void build_phase(pgc_ctx* ctx, Phase& ph, int slot) {
@@ -350,6 +410,8 @@ void build_phase(pgc_ctx* ctx, Phase& ph, int slot) {
     ph.sk_items = item;
     ph.e_item0.push_back(0);
     for (int e = 0; e < nE; ++e) ph.e_item0.push_back(ph.e_item0.back() + items_of[e]);
+  } else if (ctx->split) {
+    build_split_units(ctx, ph);
   } else {
     for (int e = 0; e <= nE; ++e) ph.e_item0.push_back(e);
     if (ctx->tc) {
@@ -428,12 +490,20 @@ cudaError_t record_event(pgc_ctx* ctx) {
   return cudaEventRecord(ctx->ev_pool[ctx->ev_used++], ctx->stream);
 }
 
+// The 16-bit copy of beta that the kernels of bf16 features (or of split
+// operands) read, from w.
+cudaError_t refresh_wb(pgc_ctx* ctx) {
+  if (ctx->split)
+    return launch_split_weights(ctx->w, ctx->wb, ctx->P, (int64_t)ctx->sp_Kp * ctx->ld, ctx->stream);
+  return launch_f32_to_bf16(ctx->w, ctx->wb, ctx->P, ctx->stream);
+}
+
 void free_all(pgc_ctx* ctx) {
   for (cudaEvent_t ev : ctx->ev_pool) cudaEventDestroy(ev);
   ctx->ev_pool.clear();
   void* ptrs[] = {ctx->X, ctx->y, ctx->w, ctx->wb, ctx->store, ctx->U, ctx->gout, ctx->partials, ctx->Z,
                   ctx->coeff, ctx->status, ctx->loss_blocks, ctx->loss_out, ctx->tables, ctx->counters, ctx->Rb,
-                  ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre};
+                  ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre, ctx->R3, ctx->tmX};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (ctx->status_h) cudaFreeHost(ctx->status_h);
@@ -519,11 +589,16 @@ int pgc_create(pgc_ctx** out, int32_t n, int32_t s, int32_t scheme, int32_t loss
   return pgc_create_mode(out, PGC_MODE_PGC, n, s, scheme, loss, dtype, d, K, rows, lr, w0, stream);
 }
 
-int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t scheme, int32_t loss,
-                    int32_t dtype, int64_t d, int64_t K, const int64_t* rows, float lr, const float* w0,
-                    void* stream) {
-  if (!out) return PGC_EINVAL;
-  *out = nullptr;
+}  // extern "C"
+
+namespace {
+
+// pgc_create_mode; *split: in, whether the single-precision tensor-core
+// softmax path may be taken; out, whether it was.
+int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t scheme, int32_t loss, int32_t dtype,
+                   int64_t d, int64_t K, const int64_t* rows, float lr, const float* w0, void* stream, bool* split) {
+  const bool allow_split = *split;
+  *split = false;
   int rc = check_nsc(scheme, n, s);
   if (rc) return rc;
   if (mode != PGC_MODE_PGC && mode != PGC_MODE_IS_SGD && mode != PGC_MODE_GC && mode != PGC_MODE_NAIVE_CR)
@@ -604,6 +679,17 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
       ctx->sk_nc = smallk_max_clusters(ctx->sk_nper);
       ctx->smallk = ctx->sk_nc > 0;
     }
+    // up to 128 classes in single precision: tensor cores on split operands
+    // (PGC_NO_SPLIT=1 keeps the CUDA-core kernels)
+    const char* env5 = std::getenv("PGC_NO_SPLIT");
+    if (!ctx->tc && !ctx->smallk && allow_split && K <= kSplitMaxClasses && !(env5 && env5[0] == '1')) {
+      ctx->sp_nc = split_max_clusters(dtype, K);
+      ctx->split = *split = ctx->sp_nc > 0;
+      ctx->sp_Kp = split_kp(K);
+      ctx->sp_C3 = split_cols(ctx->sp_Kp);
+      ctx->sp_chunk = 2;
+      if (const char* env = std::getenv("PGC_SPLIT_CHUNK")) ctx->sp_chunk = std::max(1, std::atoi(env));
+    }
   }
   ctx->P = ctx->K * ctx->ld;
   ctx->Kpad = (int64_t)align_up((size_t)K, 4);
@@ -634,6 +720,7 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
   for (auto& ph : ctx->phases) {
     // the tensor-core backward writes the stores directly: no partials
     const size_t np = ctx->tc ? 0
+                      : ctx->split ? (size_t)ph.sg_items * ctx->P
                       : ctx->smallk ? (size_t)ph.sk_items * ctx->P
                       : ctx->loss == PGC_SOFTMAX ? ph.parts.size() * (size_t)ctx->P
                                                  : ph.items.size() * (size_t)ctx->ld;
@@ -643,7 +730,7 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
   std::vector<uint8_t> tab;
   size_t off = 0;
   std::vector<size_t> offs;
-  constexpr int kTabs = 20;
+  constexpr int kTabs = 22;
   for (auto& ph : ctx->phases) {
     offs.push_back(align_up(off, 16)); put(tab, off, ph.items);
     offs.push_back(align_up(off, 16)); put(tab, off, ph.e_item0);
@@ -665,6 +752,8 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
     offs.push_back(align_up(off, 16)); put(tab, off, ph.q_tiles);
     offs.push_back(align_up(off, 16)); put(tab, off, ph.g_units);
     offs.push_back(align_up(off, 16)); put(tab, off, ph.sk_cuts);
+    offs.push_back(align_up(off, 16)); put(tab, off, ph.sl_units);
+    offs.push_back(align_up(off, 16)); put(tab, off, ph.sg_units);
   }
   // loss chunks (softmax): {row0, rows, 0} per chunk
   std::vector<int64_t> ldesc;
@@ -695,8 +784,11 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
   PGC_ALLOC(ctx->X, (size_t)ctx->total_rows * ctx->ld * ctx->esize);
   PGC_ALLOC(ctx->y, (size_t)ctx->total_rows * 4 + 64);   // per-stage label copies overrun by <= 12 B
   PGC_ALLOC(ctx->w, Pb);
-  const size_t wb_elems = ctx->tc ? (size_t)ctx->Ktc * ctx->ld : ctx->smallk ? (size_t)16 * ctx->ld : (size_t)ctx->P;
-  if (dtype == PGC_BF16) PGC_ALLOC(ctx->wb, wb_elems * 2);
+  const size_t wb_elems = ctx->tc       ? (size_t)ctx->Ktc * ctx->ld
+                          : ctx->smallk ? (size_t)16 * ctx->ld
+                          : ctx->split  ? (size_t)3 * ctx->sp_Kp * ctx->ld
+                                        : (size_t)ctx->P;
+  if (dtype == PGC_BF16 || ctx->split) PGC_ALLOC(ctx->wb, wb_elems * 2);
   PGC_ALLOC(ctx->store, (size_t)ctx->owners * ctx->c * Pb);
   PGC_ALLOC(ctx->U, (size_t)ctx->c * Pb);
   PGC_ALLOC(ctx->gout, Pb);
@@ -704,11 +796,15 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
   int64_t max_zpad = 0;
   for (auto& ph : ctx->phases) max_zpad = std::max(max_zpad, ph.zpad_total);
   if (loss == PGC_SOFTMAX) {
-    const size_t zcc = (size_t)std::max<int64_t>(max_z, ctx->loss_chunk) * ctx->Kpad;
+    const size_t zcc = (size_t)std::max<int64_t>(ctx->split ? 0 : max_z, ctx->loss_chunk) * ctx->Kpad;
     const size_t ztc = ctx->tc && !ctx->tcf ? (size_t)max_zpad * ctx->Ktc : 0;
     PGC_ALLOC(ctx->Z, std::max(zcc, ztc) * sizeof(float));
   }
   if (ctx->tc) PGC_ALLOC(ctx->Rb, (size_t)max_zpad * ctx->Ktc * sizeof(uint16_t));
+  if (ctx->split) {
+    PGC_ALLOC(ctx->R3, (size_t)max_zpad * ctx->sp_C3 * sizeof(uint16_t));
+    PGC_ALLOC(ctx->tmX, (size_t)2 * n * 128);
+  }
   // The decode's terms of the slots other than o_t are summed by four warps
   // of the fused logits kernel when that pays: the decode after the gradient
   // contraction then reads (c - 1)(1 + s) P floats less (at about 6.5 TB/s),
@@ -759,7 +855,7 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
     e = cudaMemcpy2DAsync(ctx->w, ctx->ld * sizeof(float), w0, d * sizeof(float), d * sizeof(float), K,
                           cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && ctx->wb) e = cudaMemsetAsync(ctx->wb, 0, wb_elems * 2, st);
-  if (e == cudaSuccess && ctx->wb) e = launch_f32_to_bf16(ctx->w, ctx->wb, ctx->P, st);
+  if (e == cudaSuccess && ctx->wb) e = refresh_wb(ctx);
   if (e == cudaSuccess && ctx->Rb) e = cudaMemsetAsync(ctx->Rb, 0, (size_t)max_zpad * ctx->Ktc * 2, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(e);
@@ -788,6 +884,8 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
     ph.d_q_tiles = reinterpret_cast<int32_t*>(base + o[17]);
     ph.d_g_units = reinterpret_cast<int32_t*>(base + o[18]);
     ph.d_sk_cuts = reinterpret_cast<int32_t*>(base + o[19]);
+    ph.d_sl_units = reinterpret_cast<SplitUnit*>(base + o[20]);
+    ph.d_sg_units = reinterpret_cast<SplitUnit*>(base + o[21]);
   }
   ctx->loss_desc = nullptr;
   if (!ldesc.empty()) ctx->loss_desc = reinterpret_cast<int64_t*>(base + ldesc_off);
@@ -800,6 +898,25 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
     if (!make_tmap_bf16(ctx->tmXk, ctx->X, ctx->ld, ctx->total_rows, pitch, kSmallKRows) ||
         !make_tmap_bf16(ctx->tmW16, ctx->wb, ctx->ld, 16, pitch, 16))
       return fail(cudaErrorInvalidValue);
+  }
+  if (ctx->split) {
+    // X through one map per partition: rows past it read as zero
+    const bool f32 = dtype == PGC_F32;
+    const uint64_t pitch = (uint64_t)ctx->ld * ctx->esize;
+    std::vector<uint8_t> maps((size_t)2 * n * 128 + 64);
+    uint8_t* m = reinterpret_cast<uint8_t*>(align_up(reinterpret_cast<uintptr_t>(maps.data()), 64));
+    bool ok = make_tmap_2d(ctx->tmW3, false, ctx->wb, ctx->ld, 3 * ctx->sp_Kp, (uint64_t)ctx->ld * 2, 64,
+                           (uint32_t)(3 * ctx->sp_Kp / 2), true) &&
+              make_tmap_2d(ctx->tmR3, false, ctx->R3, ctx->sp_C3, max_zpad, (uint64_t)ctx->sp_C3 * 2, 64, 32, true);
+    for (int k = 0; k < n && ok; ++k) {
+      const uint8_t* Xk = static_cast<const uint8_t*>(ctx->X) + (size_t)ctx->row0[k] * pitch;
+      ok = make_tmap_2d(m + (size_t)k * 128, f32, Xk, ctx->ld, ctx->rows[k], pitch, f32 ? 32 : 64, 128, true) &&
+           make_tmap_2d(m + (size_t)(n + k) * 128, f32, Xk, ctx->ld, ctx->rows[k], pitch, f32 ? 128 : 64, 64, !f32);
+    }
+    if (!ok) return fail(cudaErrorInvalidValue);
+    e = cudaMemcpyAsync(ctx->tmX, m, (size_t)2 * n * 128, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return fail(e);
   }
   if (ctx->tc) {
     const uint64_t pitch = (uint64_t)ctx->ld * 2;
@@ -822,6 +939,27 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
 #undef PGC_ALLOC
   *out = ctx;
   return PGC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t scheme, int32_t loss,
+                    int32_t dtype, int64_t d, int64_t K, const int64_t* rows, float lr, const float* w0,
+                    void* stream) {
+  if (!out) return PGC_EINVAL;
+  *out = nullptr;
+  bool split = true;
+  int rc = create_context(out, mode, n, s, scheme, loss, dtype, d, K, rows, lr, w0, stream, &split);
+  if (rc == PGC_ENOMEM && split) {
+    // its residual buffer is larger than the CUDA-core kernels': a run that
+    // fits only without it takes them
+    cudaGetLastError();
+    split = false;
+    rc = create_context(out, mode, n, s, scheme, loss, dtype, d, K, rows, lr, w0, stream, &split);
+  }
+  return rc;
 }
 
 int pgc_destroy(pgc_ctx* ctx) {
@@ -881,6 +1019,7 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
   DecodeArgs dc;
   dc.scheme = ctx->scheme; dc.n = n; dc.s = ctx->s; dc.c = c; dc.slot = ph.slot; dc.owners = ctx->owners;
   dc.mask = bits; dc.P = ctx->P; dc.store = ctx->store; dc.U = ctx->U; dc.w = ctx->w; dc.wb = ctx->wb;
+  dc.wb_stride = ctx->split ? (int64_t)ctx->sp_Kp * ctx->ld : 0;
   dc.gout = ctx->gout; dc.lr = ctx->lr; dc.coeff_out = ctx->coeff; dc.status = ctx->status;
   // outputs with the unpadded layout (ld == d) and 16-byte alignment that the
   // GPU can address are written by the decode itself: device outputs (so no
@@ -989,6 +1128,20 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
     a.status = ctx->status; a.pdl = ctx->pdl ? 1 : 0;
     nl[PGC_KGRAD] = 1;
     PGC_CK(ctx, launch_softmax_smallk(ctx->tmXk, ctx->tmW16, a, ctx->sk_nc, st));
+  } else if (ctx->split) {
+    SplitArgs a = {};
+    a.K = (int)ctx->K; a.Kp = ctx->sp_Kp; a.C3 = ctx->sp_C3; a.ld = ctx->ld; a.P = ctx->P;
+    a.nkb = (int)(ctx->ld / 64); a.chunk = ctx->sp_chunk;
+    a.R3 = ctx->R3; a.y = static_cast<const int32_t*>(ctx->y); a.partials = ctx->partials;
+    a.e_scale = ph.d_e_scale; a.e_dest = ph.d_e_dest; a.ndest = ph.ndest; a.store = ctx->store;
+    a.status = ctx->status;
+    a.tmX = ctx->tmX; a.units = ph.d_sl_units; a.nunits = (int)ph.sl_units.size();
+    PGC_CK(ctx, launch_split(false, ctx->dtype, ctx->tmW3, a, ctx->sp_nc, ctx->pdl, st));
+    a.tmX = static_cast<const uint8_t*>(ctx->tmX) + (size_t)n * 128;
+    a.units = ph.d_sg_units; a.nunits = (int)ph.sg_units.size();
+    PGC_CK(ctx, launch_split(true, ctx->dtype, ctx->tmR3, a, ctx->sp_nc, ctx->pdl, st));
+    nl[PGC_KGRAD] = 2;
+    need_commit = ph.sg_items > 0;
   } else {
     SoftmaxCCArgs a;
     a.dtype = ctx->dtype; a.ld = ctx->ld; a.K = ctx->K; a.X = ctx->X; a.y = static_cast<const int32_t*>(ctx->y);
@@ -1166,7 +1319,7 @@ int pgc_set_weights(pgc_ctx* ctx, const float* w) {
   if (ctx->broken) return PGC_ESTATE;
   PGC_CK(ctx, cudaMemcpy2DAsync(ctx->w, ctx->ld * sizeof(float), w, ctx->d * sizeof(float), ctx->d * sizeof(float),
                                 ctx->K, cudaMemcpyHostToDevice, ctx->stream));
-  if (ctx->wb) PGC_CK(ctx, launch_f32_to_bf16(ctx->w, ctx->wb, ctx->P, ctx->stream));
+  if (ctx->wb) PGC_CK(ctx, refresh_wb(ctx));
   return read_status(ctx);
 }
 
@@ -1228,7 +1381,7 @@ int pgc_checkpoint_load(pgc_ctx* ctx, const void* buf, int64_t bytes) {
   p += Kd;
   for (int64_t r = 0; r < (int64_t)ctx->owners * ctx->c; ++r, p += Kd) PGC_CK(ctx, copy_in(ctx->store + r * ctx->P, p));
   for (int o = 0; o < ctx->c; ++o, p += Kd) PGC_CK(ctx, copy_in(ctx->U + (int64_t)o * ctx->P, p));
-  if (ctx->wb) PGC_CK(ctx, launch_f32_to_bf16(ctx->w, ctx->wb, ctx->P, ctx->stream));
+  if (ctx->wb) PGC_CK(ctx, refresh_wb(ctx));
   const int rc = read_status(ctx);
   if (rc) return rc;
   ctx->t = h[11];

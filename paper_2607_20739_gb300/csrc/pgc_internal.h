@@ -44,6 +44,7 @@ struct DecodeArgs {
   float* U;                 // [c][P] slot totals
   float* w;                 // [P] parameters, updated in place
   uint16_t* wb;             // [P] bf16 copy of w, or nullptr
+  int64_t wb_stride = 0;    // != 0: wb holds w as three bf16 parts, this many elements apart
   float* gout;              // [P] decoded gradient
   float lr;
   float* coeff_out;         // [n] per-worker coefficient a_i (written once per step)
@@ -357,6 +358,53 @@ cudaError_t launch_softmax_rows(const void* tmX, const RowsArgs& a, int nctas, c
 // tm_out and base both nullptr it only checks that the view can be encoded.
 bool make_tmap_bf16_rows(void* tm_out, const void* base, uint64_t ld, uint64_t rows, uint32_t box_rows,
                          uint32_t box_blocks);
+
+// ---- softmax in single precision on the tensor cores (softmax_split.cu) -----
+// K <= kSplitMaxClasses classes; W and R as three bf16 parts side by side along
+// the MMA's N axis (3 Kp columns), fp32 X cut into three parts in the kernel.
+constexpr int64_t kSplitMaxClasses = 128;
+constexpr int kSplitRows = 256;            // rows of X per logits unit (two CTAs of 128)
+constexpr int kSplitFeatures = 256;        // features per gradient unit (two CTAs of 128)
+inline int split_kp(int64_t K) { return (int)((K + 15) / 16 * 16); }
+inline int split_cols(int Kp) { return (3 * Kp + 63) / 64 * 64; }   // columns of R
+struct SplitUnit {
+  int32_t e;      // position of the partition in the phase's evaluated list
+  int32_t map;    // its tensor map (partition index)
+  int32_t x;      // logits: first global row of the partition (labels); gradient: 256-feature tile
+  int32_t r0;     // first row of the unit within the partition
+  int32_t rows;   // logits: rows of the partition; gradient: rows of the unit (from r0)
+  int32_t z0;     // first R row of the partition (a multiple of 128)
+  int32_t item;   // gradient: partial that receives the sums, or -1: scaled, into the stores
+  int32_t pad;
+};
+struct SplitArgs {
+  const SplitUnit* units;
+  int nunits;
+  const void* tmX;          // device array of tensor maps, one per partition
+  int nkb;                  // logits: ld / 64
+  int chunk;                // K blocks of 64 per accumulator before it is added up in fp32
+  int K, Kp, C3;            // classes, padded to 16, columns of R (split_cols)
+  int64_t ld, P;
+  uint16_t* R3;             // residual parts [rows][C3]: r1 | r2 | r3, Kp columns each
+  const int32_t* y;         // logits: labels per global row
+  float* partials;          // gradient: [items][P]
+  const float* e_scale;     // gradient straight into the stores
+  const int32_t* e_dest;
+  int ndest;
+  float* store;
+  int* status;
+};
+// Clusters of two CTAs that fit at once, for both kernels (0: cannot launch).
+int split_max_clusters(int dtype, int64_t K);
+// grad = false: R from X and W; tmB = W parts [3 Kp][ld], box {64, 3 Kp / 2}; tmX: box
+// {128 bytes, 128} per partition, 128-byte swizzle.  grad = true: partials (or stores) from R and X;
+// tmB = R [rows][C3], box {64, 32}; tmX: bf16 box {64, 64}, 128-byte swizzle; fp32 box {128, 64}, no swizzle.
+cudaError_t launch_split(bool grad, int dtype, const void* tmB, const SplitArgs& a, int nclusters, bool pdl,
+                         cudaStream_t st);
+cudaError_t launch_split_weights(const float* src, uint16_t* dst, int64_t count, int64_t stride, cudaStream_t st);
+// 2-D tensor map [outer][inner], row pitch in bytes, box {box_inner, box_outer}, 128-byte swizzle or none
+bool make_tmap_2d(void* tm_out, bool f32, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_bytes,
+                  uint32_t box_inner, uint32_t box_outer, bool swizzle);
 
 // ---- misc -------------------------------------------------------------------
 cudaError_t launch_f32_to_bf16(const float* src, uint16_t* dst, int64_t count, cudaStream_t st);

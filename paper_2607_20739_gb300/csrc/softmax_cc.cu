@@ -1,4 +1,6 @@
-// Softmax cross-entropy partition gradient on CUDA cores, any K (§III with
+// Softmax cross-entropy partition gradient on CUDA cores, any K (more than 128
+// classes outside the bf16 tensor-core kernels; up to 128 softmax_split.cu runs
+// at 3 to 12 times the rate, unless its buffers do not fit) (§III with
 // f = log sum_k exp(w_k.x) - w_y.x):
 //   Z = X_e W^T            (tiled fp32 FMA, features widened from bf16/fp32)
 //   R = softmax(Z) - onehot(y)      (row-wise, in place)

@@ -140,6 +140,20 @@ __device__ __forceinline__ void write_coeffs_warp(const DecodeArgs& a, int lane)
     a.coeff_out[i] = cr ? (straggles(a.mask, i) ? 0.f : A) : (fr_rep(a, i / a.c) == i ? A : 0.f);
 }
 
+// Four parameters (float4 column i) as three bf16 parts each, w = w1 + w2 + w3
+// up to 2^-27 |w| (round to nearest); part j of the array starts at j * stride.
+__device__ __forceinline__ void store_split4(uint16_t* dst, int64_t stride, int64_t i, float4 v) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    uint2 pk;
+    pk.x = *reinterpret_cast<const uint32_t*>(&lo);
+    pk.y = *reinterpret_cast<const uint32_t*>(&hi);
+    reinterpret_cast<uint2*>(dst + j * stride)[i] = pk;
+    v = make_float4(v.x - __low2float(lo), v.y - __high2float(lo), v.z - __low2float(hi), v.w - __high2float(hi));
+  }
+}
+
 __device__ __forceinline__ void store_outputs(const DecodeArgs& a, int64_t p, float4 g, float4 w) {
   reinterpret_cast<float4*>(a.w)[p] = w;
   reinterpret_cast<float4*>(a.gout)[p] = g;
@@ -152,6 +166,21 @@ __device__ __forceinline__ void store_outputs(const DecodeArgs& a, int64_t p, fl
     pk.x = *reinterpret_cast<uint32_t*>(&lo);
     pk.y = *reinterpret_cast<uint32_t*>(&hi);
     reinterpret_cast<uint2*>(a.wb)[p] = pk;
+  }
+}
+
+// store_outputs for the standalone decode kernels, which also serve the path
+// whose kernels read beta as three bf16 parts (the fused tails never do, and
+// the branch there cost the few-class kernel 2 us of its 57).
+__device__ __forceinline__ void store_outputs_any(const DecodeArgs& a, int64_t p, float4 g, float4 w) {
+  if (a.wb_stride) {
+    store_split4(a.wb, a.wb_stride, p, w);
+    reinterpret_cast<float4*>(a.w)[p] = w;
+    reinterpret_cast<float4*>(a.gout)[p] = g;
+    if (a.w_user) reinterpret_cast<float4*>(a.w_user)[p] = w;
+    if (a.g_user) reinterpret_cast<float4*>(a.g_user)[p] = g;
+  } else {
+    store_outputs(a, p, g, w);
   }
 }
 
@@ -277,7 +306,7 @@ __device__ void decode_chunks(const DecodeArgs& a, const DecodePlan& pl, float4 
       const float4 g = f4fma(B, V, D);
       float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       w = f4fma(-a.lr, g, w);
-      store_outputs(a, p, g, w);
+      store_outputs_any(a, p, g, w);
     }
     bar();
   }
