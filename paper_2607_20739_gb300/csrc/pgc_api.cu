@@ -173,7 +173,13 @@ struct pgc_ctx {
   double* gc_draws = nullptr;  // [s][n-1] the construction's draws (staging)
   float* gc_wts = nullptr;     // [n][c] the last step's d_j c_{j,l} / n
   int64_t loss_chunk = 0;
-  int loss_nblocks = 256;
+  int loss_nblocks = 256;      // block sums (CTAs) of the loss kernels
+  int lw_nc = 0;               // softmax loss on the tensor cores: its clusters (0: tiled CUDA-core logits)
+  int lw_Kp = 0, lw_ncb = 0;   // its class blocks: ncb of Kp
+  uint16_t* lw = nullptr;      // W parts [ncb][3][Kp][ld] (split path: wb)
+  void* tmXl = nullptr;        // device tensor map of X over all rows
+  alignas(64) unsigned char tmWl[128];   // W parts
+  double* loss_h = nullptr;    // pinned host copy of the loss
   void* tables = nullptr;
 
   std::vector<Phase> phases;
@@ -494,7 +500,7 @@ cudaError_t record_event(pgc_ctx* ctx) {
 // operands) read, from w.
 cudaError_t refresh_wb(pgc_ctx* ctx) {
   if (ctx->split)
-    return launch_split_weights(ctx->w, ctx->wb, ctx->P, (int64_t)ctx->sp_Kp * ctx->ld, ctx->stream);
+    return launch_split_weights(ctx->w, ctx->wb, ctx->K, ctx->ld, ctx->sp_Kp, ctx->stream);
   return launch_f32_to_bf16(ctx->w, ctx->wb, ctx->P, ctx->stream);
 }
 
@@ -503,11 +509,14 @@ void free_all(pgc_ctx* ctx) {
   ctx->ev_pool.clear();
   void* ptrs[] = {ctx->X, ctx->y, ctx->w, ctx->wb, ctx->store, ctx->U, ctx->gout, ctx->partials, ctx->Z,
                   ctx->coeff, ctx->status, ctx->loss_blocks, ctx->loss_out, ctx->tables, ctx->counters, ctx->Rb,
-                  ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre, ctx->R3, ctx->tmX};
+                  ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre, ctx->R3, ctx->tmX, ctx->tmXl,
+                  ctx->lw == ctx->wb ? nullptr : ctx->lw};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (ctx->status_h) cudaFreeHost(ctx->status_h);
   ctx->status_h = nullptr;
+  if (ctx->loss_h) cudaFreeHost(ctx->loss_h);
+  ctx->loss_h = nullptr;
 }
 
 // Device address of a pinned host buffer mapped into the current device's
@@ -630,6 +639,8 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   for (int k = 0; k < n; ++k) { ctx->row0[k] = acc; acc += rows[k]; }
   ctx->total_rows = acc;
 
+  const char* env5 = std::getenv("PGC_NO_SPLIT");
+  const bool no_split = env5 && env5[0] == '1';
   if (loss != PGC_SOFTMAX) {
     ctx->variant = grad_rows_variant(dtype, d, &ctx->ld);
     if (ctx->variant < 0) { delete ctx; return PGC_ENOTSUP; }
@@ -681,14 +692,12 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     }
     // up to 128 classes in single precision: tensor cores on split operands
     // (PGC_NO_SPLIT=1 keeps the CUDA-core kernels)
-    const char* env5 = std::getenv("PGC_NO_SPLIT");
-    if (!ctx->tc && !ctx->smallk && allow_split && K <= kSplitMaxClasses && !(env5 && env5[0] == '1')) {
-      ctx->sp_nc = split_max_clusters(dtype, K);
+    if (!ctx->tc && !ctx->smallk && allow_split && K <= kSplitMaxClasses && !no_split) {
+      ctx->sp_nc = std::min(split_max_clusters(kSplitLogits, dtype, K), split_max_clusters(kSplitGrad, dtype, K));
       ctx->split = *split = ctx->sp_nc > 0;
       ctx->sp_Kp = split_kp(K);
       ctx->sp_C3 = split_cols(ctx->sp_Kp);
-      ctx->sp_chunk = 2;
-      if (const char* env = std::getenv("PGC_SPLIT_CHUNK")) ctx->sp_chunk = std::max(1, std::atoi(env));
+      ctx->sp_chunk = kSplitChunk;
     }
   }
   ctx->P = ctx->K * ctx->ld;
@@ -795,8 +804,28 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   PGC_ALLOC(ctx->partials, max_partials * sizeof(float));
   int64_t max_zpad = 0;
   for (auto& ph : ctx->phases) max_zpad = std::max(max_zpad, ph.zpad_total);
+  if (loss == PGC_SOFTMAX && !no_split && ctx->total_rows < (int64_t(1) << 31) - kSplitRows) {
+    // the loss on the tensor cores, if the parts of W fit
+    ctx->lw_nc = split_max_clusters(kSplitLoss, dtype, std::min(K, kSplitMaxClasses));
+    ctx->lw_Kp = split_kp(std::min(K, kSplitMaxClasses));
+    ctx->lw_ncb = (int)((K + ctx->lw_Kp - 1) / ctx->lw_Kp);
+    if (ctx->split) ctx->lw = ctx->wb;
+    else if (ctx->lw_nc > 0 &&
+             cudaMalloc((void**)&ctx->lw, (size_t)3 * ctx->lw_ncb * ctx->lw_Kp * ctx->ld * 2) != cudaSuccess) {
+      cudaGetLastError();
+      ctx->lw = nullptr;
+      ctx->lw_nc = 0;
+    }
+    if (ctx->lw_nc > 0) {
+      PGC_ALLOC(ctx->tmXl, 128);
+      ctx->loss_nblocks = 8 * ctx->lw_nc;
+    }
+  } else if (loss != PGC_SOFTMAX) {
+    ctx->loss_nblocks = 8 * ctx->sm_count;
+  }
   if (loss == PGC_SOFTMAX) {
-    const size_t zcc = (size_t)std::max<int64_t>(ctx->split ? 0 : max_z, ctx->loss_chunk) * ctx->Kpad;
+    const size_t zcc = (size_t)std::max<int64_t>(ctx->tc || ctx->smallk || ctx->split ? 0 : max_z,
+                                              ctx->lw_nc > 0 ? 0 : ctx->loss_chunk) * ctx->Kpad;
     const size_t ztc = ctx->tc && !ctx->tcf ? (size_t)max_zpad * ctx->Ktc : 0;
     PGC_ALLOC(ctx->Z, std::max(zcc, ztc) * sizeof(float));
   }
@@ -827,6 +856,8 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   {
     cudaError_t _e = cudaMallocHost((void**)&ctx->status_h, sizeof(int));
     if (_e != cudaSuccess) return fail(_e);
+    _e = cudaMallocHost((void**)&ctx->loss_h, sizeof(double));
+    if (_e != cudaSuccess) return fail(_e);
   }
   PGC_ALLOC(ctx->loss_blocks, (size_t)ctx->loss_nblocks * sizeof(double));
   PGC_ALLOC(ctx->loss_out, sizeof(double));
@@ -856,6 +887,8 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
                           cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && ctx->wb) e = cudaMemsetAsync(ctx->wb, 0, wb_elems * 2, st);
   if (e == cudaSuccess && ctx->wb) e = refresh_wb(ctx);
+  if (e == cudaSuccess && ctx->lw && ctx->lw != ctx->wb)
+    e = cudaMemsetAsync(ctx->lw, 0, (size_t)3 * ctx->lw_ncb * ctx->lw_Kp * ctx->ld * 2, st);
   if (e == cudaSuccess && ctx->Rb) e = cudaMemsetAsync(ctx->Rb, 0, (size_t)max_zpad * ctx->Ktc * 2, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(e);
@@ -898,6 +931,17 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     if (!make_tmap_bf16(ctx->tmXk, ctx->X, ctx->ld, ctx->total_rows, pitch, kSmallKRows) ||
         !make_tmap_bf16(ctx->tmW16, ctx->wb, ctx->ld, 16, pitch, 16))
       return fail(cudaErrorInvalidValue);
+  }
+  if (ctx->lw_nc > 0) {
+    alignas(64) unsigned char m[128];
+    const bool f32 = dtype == PGC_F32;
+    if (!make_tmap_2d(ctx->tmWl, false, ctx->lw, ctx->ld, (uint64_t)3 * ctx->lw_ncb * ctx->lw_Kp, (uint64_t)ctx->ld * 2, 64,
+                      (uint32_t)(3 * ctx->lw_Kp / 2), true) ||
+        !make_tmap_2d(m, f32, ctx->X, ctx->ld, ctx->total_rows, (uint64_t)ctx->ld * ctx->esize, f32 ? 32 : 64, 128, true))
+      return fail(cudaErrorInvalidValue);
+    e = cudaMemcpyAsync(ctx->tmXl, m, 128, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return fail(e);
   }
   if (ctx->split) {
     // X through one map per partition: rows past it read as zero
@@ -1136,10 +1180,10 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
     a.e_scale = ph.d_e_scale; a.e_dest = ph.d_e_dest; a.ndest = ph.ndest; a.store = ctx->store;
     a.status = ctx->status;
     a.tmX = ctx->tmX; a.units = ph.d_sl_units; a.nunits = (int)ph.sl_units.size();
-    PGC_CK(ctx, launch_split(false, ctx->dtype, ctx->tmW3, a, ctx->sp_nc, ctx->pdl, st));
+    PGC_CK(ctx, launch_split(kSplitLogits, ctx->dtype, ctx->tmW3, a, ctx->sp_nc, ctx->pdl, st));
     a.tmX = static_cast<const uint8_t*>(ctx->tmX) + (size_t)n * 128;
     a.units = ph.d_sg_units; a.nunits = (int)ph.sg_units.size();
-    PGC_CK(ctx, launch_split(true, ctx->dtype, ctx->tmR3, a, ctx->sp_nc, ctx->pdl, st));
+    PGC_CK(ctx, launch_split(kSplitGrad, ctx->dtype, ctx->tmR3, a, ctx->sp_nc, ctx->pdl, st));
     nl[PGC_KGRAD] = 2;
     need_commit = ph.sg_items > 0;
   } else {
@@ -1216,14 +1260,29 @@ int pgc_sync(pgc_ctx* ctx) {
 int pgc_loss(pgc_ctx* ctx, double* loss_out) {
   if (!ctx || !loss_out) return PGC_EINVAL;
   if (!ctx->loaded || ctx->broken) return PGC_ESTATE;
-  LossArgs a;
-  a.loss = ctx->loss; a.dtype = ctx->dtype; a.ld = ctx->ld; a.K = ctx->K; a.rows = ctx->total_rows;
-  a.X = ctx->X; a.y = ctx->y; a.w = ctx->w; a.blocksum = ctx->loss_blocks; a.nblocks = ctx->loss_nblocks;
-  a.out = ctx->loss_out; a.Z = ctx->Z; a.Kpad = ctx->Kpad; a.z_chunk_rows = ctx->loss_chunk;
-  a.chunk_desc = ctx->loss_desc;
-  PGC_CK(ctx, launch_loss(a, ctx->stream));
-  PGC_CK(ctx, cudaMemcpyAsync(loss_out, ctx->loss_out, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-  return read_status(ctx);
+  if (ctx->lw_nc > 0) {
+    if (ctx->lw != ctx->wb) PGC_CK(ctx, launch_split_weights(ctx->w, ctx->lw, ctx->K, ctx->ld, ctx->lw_Kp, ctx->stream));
+    SplitArgs a = {};
+    a.K = (int)ctx->K; a.Kp = ctx->lw_Kp; a.ncb = ctx->lw_ncb; a.ld = ctx->ld; a.nkb = (int)(ctx->ld / 64);
+    a.chunk = kSplitChunk; a.tmX = ctx->tmXl; a.rows = ctx->total_rows; a.blocksum = ctx->loss_blocks;
+    a.nunits = (int)((ctx->total_rows + kSplitRows - 1) / kSplitRows);
+    a.y = static_cast<const int32_t*>(ctx->y); a.status = ctx->status;
+    PGC_CK(ctx, launch_split(kSplitLoss, ctx->dtype, ctx->tmWl, a, ctx->lw_nc, false, ctx->stream));
+    PGC_CK(ctx, launch_loss_finish(ctx->loss_blocks, 8 * std::min(a.nunits, ctx->lw_nc), ctx->total_rows, ctx->loss_out,
+                                   ctx->stream));
+  } else {
+    LossArgs a;
+    a.loss = ctx->loss; a.dtype = ctx->dtype; a.ld = ctx->ld; a.K = ctx->K; a.rows = ctx->total_rows;
+    a.X = ctx->X; a.y = ctx->y; a.w = ctx->w; a.blocksum = ctx->loss_blocks; a.nblocks = ctx->loss_nblocks;
+    a.out = ctx->loss_out; a.Z = ctx->Z; a.Kpad = ctx->Kpad; a.z_chunk_rows = ctx->loss_chunk;
+    a.chunk_desc = ctx->loss_desc;
+    PGC_CK(ctx, launch_loss(a, ctx->stream));
+  }
+  // into pinned memory: one wait for the loss and the status word
+  PGC_CK(ctx, cudaMemcpyAsync(ctx->loss_h, ctx->loss_out, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+  const int rc = read_status(ctx);
+  if (rc == PGC_OK) *loss_out = *ctx->loss_h;
+  return rc;
 }
 
 int pgc_get_store(pgc_ctx* ctx, int32_t worker, int32_t slot, float* out) {

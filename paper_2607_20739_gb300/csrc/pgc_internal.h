@@ -176,6 +176,8 @@ struct LossArgs {
   const int64_t* chunk_desc; // device [3 * nchunks]: {row0, rows, 0} per chunk
 };
 cudaError_t launch_loss(const LossArgs& a, cudaStream_t st);
+// out = (sum of blocksum) / rows
+cudaError_t launch_loss_finish(const double* blocksum, int nblocks, int64_t rows, double* out, cudaStream_t st);
 
 // ---- tensor-core logits GEMM (tc_gemm.cu) --------------------------------
 // Z[r][k] = sum_j X[r][j] Wb[k][j] (A = X K-major, B = Wb K-major), for the
@@ -363,6 +365,8 @@ bool make_tmap_bf16_rows(void* tm_out, const void* base, uint64_t ld, uint64_t r
 // K <= kSplitMaxClasses classes; W and R as three bf16 parts side by side along
 // the MMA's N axis (3 Kp columns), fp32 X cut into three parts in the kernel.
 constexpr int64_t kSplitMaxClasses = 128;
+enum { kSplitLogits = 0, kSplitGrad = 1, kSplitLoss = 2 };   // kernels (launch_split's mode)
+constexpr int kSplitChunk = 2;             // 64-wide K blocks per leading accumulator
 constexpr int kSplitRows = 256;            // rows of X per logits unit (two CTAs of 128)
 constexpr int kSplitFeatures = 256;        // features per gradient unit (two CTAs of 128)
 inline int split_kp(int64_t K) { return (int)((K + 15) / 16 * 16); }
@@ -393,15 +397,22 @@ struct SplitArgs {
   int ndest;
   float* store;
   int* status;
+  // loss: row tiles nunits = ceil(rows / 256) of one map over all rows, ncb
+  // blocks of Kp classes; per epilogue warp of every CTA one sum of log sum exp - z_y
+  int64_t rows;
+  int ncb;
+  double* blocksum;         // [4 x CTAs]
 };
-// Clusters of two CTAs that fit at once, for both kernels (0: cannot launch).
-int split_max_clusters(int dtype, int64_t K);
-// grad = false: R from X and W; tmB = W parts [3 Kp][ld], box {64, 3 Kp / 2}; tmX: box
-// {128 bytes, 128} per partition, 128-byte swizzle.  grad = true: partials (or stores) from R and X;
+// Clusters of two CTAs that fit at once (0: cannot launch).
+int split_max_clusters(int mode, int dtype, int64_t K);
+// kSplitLogits: R from X and W; tmB = W parts [3 Kp][ld], box {64, 3 Kp / 2}; tmX: box
+// {128 bytes, 128} per partition, 128-byte swizzle.  kSplitGrad: partials (or stores) from R and X;
 // tmB = R [rows][C3], box {64, 32}; tmX: bf16 box {64, 64}, 128-byte swizzle; fp32 box {128, 64}, no swizzle.
-cudaError_t launch_split(bool grad, int dtype, const void* tmB, const SplitArgs& a, int nclusters, bool pdl,
+// kSplitLoss: tmB = W parts [ncb][3 Kp][ld]; tmX: one map over all rows, box as kSplitLogits.
+cudaError_t launch_split(int mode, int dtype, const void* tmB, const SplitArgs& a, int nclusters, bool pdl,
                          cudaStream_t st);
-cudaError_t launch_split_weights(const float* src, uint16_t* dst, int64_t count, int64_t stride, cudaStream_t st);
+// w [K][ld] -> parts [ceil(K / Kp)][3][Kp][ld] (rows past K are not written)
+cudaError_t launch_split_weights(const float* src, uint16_t* dst, int64_t K, int64_t ld, int Kp, cudaStream_t st);
 // 2-D tensor map [outer][inner], row pitch in bytes, box {box_inner, box_outer}, 128-byte swizzle or none
 bool make_tmap_2d(void* tm_out, bool f32, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_bytes,
                   uint32_t box_inner, uint32_t box_outer, bool swizzle);

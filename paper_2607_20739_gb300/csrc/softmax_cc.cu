@@ -274,18 +274,42 @@ cudaError_t launch_softmax_cc(const SoftmaxCCArgs& a, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // Full loss F(beta) = (1 / rows) sum f (§III), fp64 accumulation.
 // ---------------------------------------------------------------------------
+// Logistic and least squares: one warp per row, four 16-byte chunks (bf16: eight
+// elements each) of the row per lane in flight.
 template <typename T>
-__global__ void loss_rows_kernel(LossArgs a) {
-  __shared__ double red[32];
+__global__ void __launch_bounds__(256) loss_rows_kernel(LossArgs a) {
+  constexpr int VEC = 16 / (int)sizeof(T), kFly = 4;
+  using V = Vec<T, VEC>;
+  __shared__ double red[8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const T* X = static_cast<const T*>(a.X);
   const float* y = static_cast<const float*>(a.y);
+  const int64_t nv = a.ld / VEC;                       // ld is a multiple of VEC
   double acc = 0.0;
   for (int64_t r = warp; r < a.rows; r += nwarps) {
+    const typename V::raw* x = reinterpret_cast<const typename V::raw*>(static_cast<const T*>(a.X) + r * a.ld);
     float dot = 0.f;
-    for (int64_t j = lane; j < a.ld; j += 32) dot = fmaf(ldx<T>(X + r * a.ld + j), a.w[j], dot);
+    for (int64_t j0 = lane; j0 < nv; j0 += 32 * kFly) {
+      typename V::raw v[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u)
+        if (j0 + 32 * u < nv) v[u] = __ldcs(x + j0 + 32 * u);
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        if (j0 + 32 * u < nv) {
+          float f[VEC];
+          V::widen(v[u], f);
+          const float4* w = reinterpret_cast<const float4*>(a.w) + (j0 + 32 * u) * (VEC / 4);
+#pragma unroll
+          for (int q = 0; q < VEC / 4; ++q) {
+            const float4 wq = w[q];
+            dot = fmaf(f[4 * q], wq.x, dot); dot = fmaf(f[4 * q + 1], wq.y, dot);
+            dot = fmaf(f[4 * q + 2], wq.z, dot); dot = fmaf(f[4 * q + 3], wq.w, dot);
+          }
+        }
+      }
+    }
     dot = warp_sum(dot);
     if (lane == 0) {
       const double z = dot, yy = y[r];
@@ -298,7 +322,7 @@ __global__ void loss_rows_kernel(LossArgs a) {
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
+    for (int i = 0; i < 8; ++i) s += red[i];
     a.blocksum[blockIdx.x] = s;
   }
 }
@@ -330,12 +354,18 @@ __global__ void loss_softmax_rows(const float* __restrict__ Z, int64_t Kpad, int
   }
 }
 
+// one warp, a fixed order
 __global__ void loss_finish(const double* blocksum, int nblocks, int64_t rows, double* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < nblocks; ++i) s += blocksum[i];
-    *out = s / (double)rows;
-  }
+  double s = 0.0;
+  for (int i = threadIdx.x; i < nblocks; i += 32) s += blocksum[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) *out = s / (double)rows;
+}
+
+cudaError_t launch_loss_finish(const double* blocksum, int nblocks, int64_t rows, double* out, cudaStream_t st) {
+  loss_finish<<<1, 32, 0, st>>>(blocksum, nblocks, rows, out);
+  return cudaGetLastError();
 }
 
 __global__ void zero_doubles(double* p, int n) {
@@ -367,8 +397,7 @@ cudaError_t launch_loss(const LossArgs& a, cudaStream_t st) {
       if (e != cudaSuccess) return e;
     }
   }
-  loss_finish<<<1, 32, 0, st>>>(a.blocksum, a.nblocks, a.rows, a.out);
-  return cudaGetLastError();
+  return launch_loss_finish(a.blocksum, a.nblocks, a.rows, a.out, st);
 }
 
 }  // namespace pgc
