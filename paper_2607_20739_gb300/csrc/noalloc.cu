@@ -96,8 +96,8 @@ extern "C" int pgc_gradient_noalloc(int32_t loss, int32_t dtype, int64_t m, int6
   if (reinterpret_cast<uintptr_t>(X) % 16 != 0 || reinterpret_cast<uintptr_t>(g_out) % 16 != 0)
     return PGC_EINVAL;
   int64_t ld = 0;
-  const int variant = pgc::grad_rows_variant(dtype, d, &ld);
-  if (variant < 0 || ld != d) return PGC_ENOTSUP;   // rows must need no padding
+  const int variant = pgc::grad_rows_variant(dtype, d, m / 148, &ld);
+  if (variant < 0 || ld != d || !pgc::grad_rows_unpadded(dtype, d)) return PGC_ENOTSUP;   // the documented row lengths
 
   unsigned char* scratch = nullptr;
   int rc = scratch_address(&scratch);

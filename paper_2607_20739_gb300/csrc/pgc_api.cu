@@ -34,6 +34,8 @@ struct Phase {
   std::vector<int32_t> parts;           // evaluated partitions (e -> k)
   std::vector<WorkItem> items;          // row-kernel work items
   std::vector<int32_t> e_item0;         // CSR of items (or one per e)
+  std::vector<int32_t> cta_item0;       // row kernel: CSR of items over the CTAs (empty: taken dynamically)
+  int32_t* d_cta_item0 = nullptr;
   std::vector<float> e_scale;           // 1 / m_e
   std::vector<int32_t> e_dest;          // [nE * ndest] store index owner*c+slot
   int ndest = 1;
@@ -226,6 +228,106 @@ int read_status(pgc_ctx* ctx) {
   return PGC_OK;
 }
 
+void add_item(pgc_ctx* ctx, Phase& ph, int e, int64_t r0, int64_t rows) {
+  WorkItem it;
+  it.e = e;
+  it.part = ph.parts[e];
+  it.row0 = ph.e_row0[e] + r0;
+  it.rows = rows;
+  ph.items.push_back(it);
+  ph.max_item_rows = std::max<int>(ph.max_item_rows, (int)rows);
+}
+
+// Rows of the streaming kernel, static: every CTA takes one run of the
+// evaluated rows in partition order, an item per partition it touches.  A CTA
+// costs its rows plus h for every item (its end costs about as long as
+// streaming 48 KB); the runs are filled to the smallest cost that covers all
+// rows with one CTA per SM, none shorter than a batch for every team of warps
+// unless a partition ends there.  Runs that end with the partition leave up to
+// 16 % of the SMs idle (64 partitions: two items each, 128 CTAs); that costs
+// where a CTA's latency bounds the kernel (32 x 2 GB in bf16, d = 1024, 3001,
+// 16384: 292, 368, 409 us per step against 277, 317, 350 with runs across
+// partitions; fp32, d = 3001: 311 against 300), and pays for fp32 rows from
+// 16 KB on, which 128 SMs stream at the HBM rate with fewer streams (d = 8192: 283
+// against 297; 64 x 2048 x 16384: 1225 against 1264).
+void build_row_ranges(pgc_ctx* ctx, Phase& ph) {
+  const int nE = (int)ph.parts.size();
+  const int64_t least = grad_rows_min_item(ctx->variant);
+  const int64_t h = std::max<int64_t>(1, 49152 / (ctx->ld * (int64_t)ctx->esize));
+  const bool cross = ctx->dtype == PGC_BF16 || ctx->ld * (int64_t)ctx->esize < 16384;
+  std::vector<int64_t> run;                 // e, first row, rows of every item; -1: next CTA
+  auto fill = [&](int64_t C) {
+    run.clear();
+    int e = 0;
+    int64_t r = 0;
+    for (int cta = 0; cta < ctx->sm_count && e < nE; ++cta) {
+      int64_t used = 0;
+      while (e < nE) {
+        const int64_t rem = ph.e_rows[e] - r, room = C - used - h;
+        if (used > 0 && room < std::min(rem, least)) break;
+        const int64_t take = std::min(rem, std::max<int64_t>(room, 1));
+        run.insert(run.end(), {e, r, take});
+        used += take + h;
+        r += take;
+        if (r == ph.e_rows[e]) {
+          ++e;
+          r = 0;
+          if (!cross) break;
+        }
+      }
+      run.push_back(-1);
+    }
+    return e == nE;
+  };
+  int64_t lo = least + h, hi = lo;
+  for (int e = 0; e < nE; ++e) hi += ph.e_rows[e] + h;
+  while (lo < hi) {
+    const int64_t mid = lo + (hi - lo) / 2;
+    if (fill(mid)) hi = mid; else lo = mid + 1;
+  }
+  fill(lo);
+  ph.e_item0.assign(nE + 1, 0);
+  ph.cta_item0.push_back(0);
+  for (size_t i = 0; i < run.size();) {
+    if (run[i] < 0) {
+      ph.cta_item0.push_back((int32_t)ph.items.size());
+      ++i;
+    } else {
+      add_item(ctx, ph, (int)run[i], run[i + 1], run[i + 2]);
+      ++ph.e_item0[run[i] + 1];
+      i += 3;
+    }
+  }
+  for (int e = 0; e < nE; ++e) ph.e_item0[e + 1] += ph.e_item0[e];
+}
+
+// The dynamic form (PGC_ITEMS_PER_SM): items of (nearly) one length L for
+// every partition, the smallest L whose item count fits per_sm waves of the
+// grid; CTAs take the items beyond the first wave as they get free.
+void build_dynamic_items(pgc_ctx* ctx, Phase& ph, int per_sm) {
+  const int nE = (int)ph.parts.size();
+  const int64_t G = (int64_t)ctx->sm_count * per_sm, least = grad_rows_min_item(ctx->variant);
+  auto items_of = [&](int e, int64_t L) {
+    return std::min(std::max<int64_t>(1, ph.e_rows[e] / least), std::max<int64_t>(1, (ph.e_rows[e] + L - 1) / L));
+  };
+  auto count = [&](int64_t L) {
+    int64_t tot = 0;
+    for (int e = 0; e < nE; ++e) tot += items_of(e, L);
+    return tot;
+  };
+  int64_t lo = 1, hi = std::max<int64_t>(1, ph.max_rows);   // count(max_rows) = nE: the fewest items possible
+  while (lo < hi) {
+    const int64_t mid = lo + (hi - lo) / 2;
+    if (count(mid) <= G) hi = mid; else lo = mid + 1;
+  }
+  ph.e_item0.push_back(0);
+  for (int e = 0; e < nE; ++e) {
+    const int64_t m = ph.e_rows[e], q = items_of(e, lo);
+    for (int64_t i = 0; i < q; ++i) add_item(ctx, ph, e, m * i / q, m * (i + 1) / q - m * i / q);
+    ph.e_item0.push_back((int32_t)ph.items.size());
+  }
+}
+
 // Units of the single-precision tensor-core softmax kernels.  Logits: 256
 // rows of a partition.  Gradient: 256 features of a run of L rows of a
 // partition; L is the multiple of 64 that minimises the rounds over the
@@ -311,48 +413,10 @@ void build_phase(pgc_ctx* ctx, Phase& ph, int slot) {
   }
   ph.z_total = R;
   if (ctx->loss != PGC_SOFTMAX) {
-    // work items per SM (default 1: one balanced static item per CTA; more are
-    // taken dynamically by the persistent grid);
-    // an item holds at least one stage of rows.  PGC_ITEMS_PER_SM overrides.
-    int per_sm = 1;
-    if (const char* env = std::getenv("PGC_ITEMS_PER_SM")) per_sm = std::max(1, std::atoi(env));
-    const int64_t G = (int64_t)ctx->sm_count * per_sm;
-    const int64_t min_rows = grad_rows_stage_rows(ctx->variant, ctx->ld, ctx->dtype);
-    // items of (nearly) one length L for every partition: the smallest L whose
-    // item count fits one wave of the grid, so that all CTAs finish together
-    // (items of unequal length leave the long ones to fewer CTAs at the end)
-    std::vector<int64_t> qe(nE), cap(nE);
-    int64_t mmax = 1;
-    for (int e = 0; e < nE; ++e) {
-      cap[e] = std::max<int64_t>(1, ph.e_rows[e] / min_rows);
-      mmax = std::max(mmax, ph.e_rows[e]);
-    }
-    auto count = [&](int64_t L) {
-      int64_t tot = 0;
-      for (int e = 0; e < nE; ++e) tot += std::min(cap[e], std::max<int64_t>(1, (ph.e_rows[e] + L - 1) / L));
-      return tot;
-    };
-    int64_t lo = 1, hi = mmax;                 // count(mmax) = nE: the fewest items possible
-    while (lo < hi) {
-      const int64_t mid = lo + (hi - lo) / 2;
-      if (count(mid) <= G) hi = mid; else lo = mid + 1;
-    }
-    for (int e = 0; e < nE; ++e) qe[e] = std::min(cap[e], std::max<int64_t>(1, (ph.e_rows[e] + lo - 1) / lo));
-    ph.e_item0.push_back(0);
-    for (int e = 0; e < nE; ++e) {
-      const int64_t m = ph.e_rows[e];
-      const int64_t q = qe[e];
-      for (int64_t i = 0; i < q; ++i) {
-        const int64_t a = m * i / q, b = m * (i + 1) / q;
-        WorkItem it;
-        it.e = e;
-        it.part = ph.parts[e];
-        it.row0 = ph.e_row0[e] + a;
-        it.rows = b - a;
-        ph.items.push_back(it);
-        ph.max_item_rows = std::max<int>(ph.max_item_rows, (int)(b - a));
-      }
-      ph.e_item0.push_back((int32_t)ph.items.size());
+    if (std::getenv("PGC_ITEMS_PER_SM")) {
+      build_dynamic_items(ctx, ph, std::max(1, std::atoi(std::getenv("PGC_ITEMS_PER_SM"))));
+    } else {
+      build_row_ranges(ctx, ph);
     }
   } else if (ctx->smallk) {
     // tiles of tr rows in partition order; cluster (whole-row variant: CTA)
@@ -642,7 +706,8 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   const char* env5 = std::getenv("PGC_NO_SPLIT");
   const bool no_split = env5 && env5[0] == '1';
   if (loss != PGC_SOFTMAX) {
-    ctx->variant = grad_rows_variant(dtype, d, &ctx->ld);
+    const int64_t rows_eval = scheme == PGC_FR ? ctx->total_rows / ctx->c : ctx->total_rows;
+    ctx->variant = grad_rows_variant(dtype, d, rows_eval / 152, &ctx->ld);
     if (ctx->variant < 0) { delete ctx; return PGC_ENOTSUP; }
   } else {
     // bf16 softmax runs on the tensor cores (PGC_NO_TC=1 keeps the CUDA-core path)
@@ -739,7 +804,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   std::vector<uint8_t> tab;
   size_t off = 0;
   std::vector<size_t> offs;
-  constexpr int kTabs = 22;
+  constexpr int kTabs = 23;
   for (auto& ph : ctx->phases) {
     offs.push_back(align_up(off, 16)); put(tab, off, ph.items);
     offs.push_back(align_up(off, 16)); put(tab, off, ph.e_item0);
@@ -763,6 +828,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     offs.push_back(align_up(off, 16)); put(tab, off, ph.sk_cuts);
     offs.push_back(align_up(off, 16)); put(tab, off, ph.sl_units);
     offs.push_back(align_up(off, 16)); put(tab, off, ph.sg_units);
+    offs.push_back(align_up(off, 16)); put(tab, off, ph.cta_item0);
   }
   // loss chunks (softmax): {row0, rows, 0} per chunk
   std::vector<int64_t> ldesc;
@@ -919,6 +985,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     ph.d_sk_cuts = reinterpret_cast<int32_t*>(base + o[19]);
     ph.d_sl_units = reinterpret_cast<SplitUnit*>(base + o[20]);
     ph.d_sg_units = reinterpret_cast<SplitUnit*>(base + o[21]);
+    if (!ph.cta_item0.empty()) ph.d_cta_item0 = reinterpret_cast<int32_t*>(base + o[22]);
   }
   ctx->loss_desc = nullptr;
   if (!ldesc.empty()) ctx->loss_desc = reinterpret_cast<int64_t*>(base + ldesc_off);
@@ -1091,7 +1158,12 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
     g.tail = ph.tail; g.pdl = ctx->pdl;
     g.prefetch_bytes = ctx->prefetch_bytes;
     g.cnt_e = ctx->counters; g.cnt_all = ctx->counters + n;
-    g.work_ctr = ctx->counters + n + 1; g.prod_done = ctx->counters + n + 2; g.grid = ctx->sm_count;
+    g.cta_item0 = ph.d_cta_item0;
+    if (g.cta_item0) {
+      g.grid = (int)ph.cta_item0.size() - 1;
+    } else {
+      g.work_ctr = ctx->counters + n + 1; g.prod_done = ctx->counters + n + 2; g.grid = ctx->sm_count;
+    }
     g.e_item0 = ph.d_e_item0; g.e_scale = ph.d_e_scale; g.e_dest = ph.d_e_dest; g.ndest = ph.ndest;
     g.nE = (int)ph.parts.size(); g.store = ctx->store; g.dec = dc;
     nl[PGC_KGRAD] = 1;

@@ -71,9 +71,11 @@ struct GradRowsArgs {
   float* partials;          // [nitems][ld]
   // Labels are copied per stage from a 16-byte aligned start, so up to 12
   // bytes past the last label are read: y must be padded by 16 bytes.
-  // Dynamic scheduling: with work_ctr set, `grid` persistent CTAs take items
+  // Static ranges: with cta_item0 [grid + 1] set, CTA b takes items
+  // cta_item0[b] .. cta_item0[b + 1] - 1.  Dynamic scheduling: with work_ctr set, `grid` persistent CTAs take items
   // blockIdx.x, then gridDim.x + atomicAdd(work_ctr, 1); the last producer
-  // resets work_ctr and prod_done.  Without it, one CTA per item.
+  // resets work_ctr and prod_done.  Without either, one CTA per item.
+  const int32_t* cta_item0 = nullptr;
   int* work_ctr = nullptr;
   int* prod_done = nullptr;
   int grid = 0;
@@ -95,7 +97,11 @@ struct GradRowsArgs {
   DecodeArgs dec;           // used when tail == 2
   int64_t prefetch_bytes = 0; // L2 warm-up per CTA before waiting for the previous step
 };
-int grad_rows_variant(int dtype, int64_t d, int64_t* ld_out);  // chooses ld, returns variant id
+// chooses the row pitch, returns the variant id (-1: rows too long);
+// rows_per_sm: rows an SM gets per launch
+int grad_rows_variant(int dtype, int64_t d, int64_t rows_per_sm, int64_t* ld_out);
+int grad_rows_min_item(int variant);   // rows that give every team of warps one batch
+bool grad_rows_unpadded(int dtype, int64_t d);   // d is a row length pgc_gradient_noalloc documents
 int grad_rows_stage_rows(int variant, int64_t ld, int dtype);
 cudaError_t launch_grad_rows(const GradRowsArgs& a, int variant, cudaStream_t st);
 
