@@ -146,7 +146,7 @@ struct pgc_ctx {
   int64_t Ktc = 0;           // classes padded to the forward N tile (256)
   uint16_t* Rb = nullptr;    // bf16 residuals [zpad rows][Ktc]
   float* pre = nullptr;      // fused tensor-core path: the decode's early terms [P]
-  int* status_h = nullptr;   // pinned host copy of the status word
+  int* status_h = nullptr;   // pinned host copy of the status word (or the word itself: status == status_h)
   alignas(64) unsigned char tmXk[128];   // X as K-major A   (box 64 x 128)
   alignas(64) unsigned char tmW[128];    // Wb as K-major B  (box 64 x 128: one CTA's half of a 256 tile)
   alignas(64) unsigned char tmR[128];    // R as MN-major A  (box 64 x 64)
@@ -214,13 +214,14 @@ int cuda_fail(pgc_ctx* ctx, cudaError_t e) {
     if (_e != cudaSuccess) return cuda_fail(ctx, _e); \
   } while (0)
 
-// Read and clear nothing: map the device status word to a code.
+// Wait for the stream and map the status word to a code.
 int read_status(pgc_ctx* ctx) {
-  // into pinned memory: the copy is a plain asynchronous one, no staging
-  cudaError_t e = cudaMemcpyAsync(ctx->status_h, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+  cudaError_t e = cudaSuccess;
+  if (ctx->status != ctx->status_h)   // else the kernels set it in the pinned word itself
+    e = cudaMemcpyAsync(ctx->status_h, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
-  const int h = *ctx->status_h;
+  const int h = *static_cast<volatile int*>(ctx->status_h);
   if (h & kErrWaitTimeout) { ctx->broken = true; return PGC_ETIMEOUT; }
   if (h & kErrBadMask) { ctx->broken = true; return PGC_EMASK; }
   if (h & kErrSingular) { ctx->broken = true; return PGC_ESINGULAR; }
@@ -572,7 +573,7 @@ void free_all(pgc_ctx* ctx) {
   for (cudaEvent_t ev : ctx->ev_pool) cudaEventDestroy(ev);
   ctx->ev_pool.clear();
   void* ptrs[] = {ctx->X, ctx->y, ctx->w, ctx->wb, ctx->store, ctx->U, ctx->gout, ctx->partials, ctx->Z,
-                  ctx->coeff, ctx->status, ctx->loss_blocks, ctx->loss_out, ctx->tables, ctx->counters, ctx->Rb,
+                  ctx->coeff, ctx->status == ctx->status_h ? nullptr : ctx->status, ctx->loss_blocks, ctx->loss_out, ctx->tables, ctx->counters, ctx->Rb,
                   ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre, ctx->R3, ctx->tmX, ctx->tmXl,
                   ctx->lw == ctx->wb ? nullptr : ctx->lw};
   for (void* p : ptrs)
@@ -918,12 +919,22 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     if (on) PGC_ALLOC(ctx->pre, Pb);
   }
   PGC_ALLOC(ctx->coeff, (size_t)n * sizeof(float));
-  PGC_ALLOC(ctx->status, sizeof(int));
   {
     cudaError_t _e = cudaMallocHost((void**)&ctx->status_h, sizeof(int));
     if (_e != cudaSuccess) return fail(_e);
     _e = cudaMallocHost((void**)&ctx->loss_h, sizeof(double));
     if (_e != cudaSuccess) return fail(_e);
+    // Kernels touch the status word only when something failed (an atomic OR).
+    // Where the GPU's atomics work on host memory, the word is the pinned one,
+    // and no copy follows a step whose caller waits.
+    *ctx->status_h = 0;
+    int native = 0;
+    void* dev = nullptr;
+    cudaDeviceGetAttribute(&native, cudaDevAttrHostNativeAtomicSupported, ctx->device);
+    if (native && cudaHostGetDevicePointer(&dev, ctx->status_h, 0) == cudaSuccess && dev == ctx->status_h)
+      ctx->status = ctx->status_h;
+    else
+      PGC_ALLOC(ctx->status, sizeof(int));
   }
   PGC_ALLOC(ctx->loss_blocks, (size_t)ctx->loss_nblocks * sizeof(double));
   PGC_ALLOC(ctx->loss_out, sizeof(double));
@@ -944,7 +955,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->U, 0, (size_t)ctx->c * Pb, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->gout, 0, Pb, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->coeff, 0, (size_t)n * sizeof(float), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->status, 0, sizeof(int), st);
+  if (e == cudaSuccess && ctx->status != ctx->status_h) e = cudaMemsetAsync(ctx->status, 0, sizeof(int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->counters, 0, (size_t)(n + 3) * sizeof(int), st);
   if (e == cudaSuccess && gc_weighted) e = cudaMemsetAsync(ctx->gc_wts, 0, (size_t)n * ctx->c * sizeof(float), st);
   if (e == cudaSuccess && gc_weighted) e = cudaMemsetAsync(ctx->gc_d, 0, (size_t)(n + 2) * sizeof(double), st);
@@ -1132,21 +1143,29 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
   dc.mask = bits; dc.P = ctx->P; dc.store = ctx->store; dc.U = ctx->U; dc.w = ctx->w; dc.wb = ctx->wb;
   dc.wb_stride = ctx->split ? (int64_t)ctx->sp_Kp * ctx->ld : 0;
   dc.gout = ctx->gout; dc.lr = ctx->lr; dc.coeff_out = ctx->coeff; dc.status = ctx->status;
-  // outputs with the unpadded layout (ld == d) and 16-byte alignment that the
-  // GPU can address are written by the decode itself: device outputs (so no
-  // copy sits between consecutive steps), and pinned host outputs mapped into
-  // the device's address space (so no device-to-host copies follow the decode)
+  // Outputs that the GPU can address (device memory, and pinned host memory
+  // mapped into the device's address space) are written by the decode itself,
+  // without the padding of the parameter rows: no copies follow it.  One class,
+  // or rows without padding: the parameters' own layout up to d (16-byte aligned);
+  // else row by row.
   float* g_dev = grad_out;
   float* w_dev = w_out;
-  bool direct = ctx->ld == ctx->d && (reinterpret_cast<uintptr_t>(grad_out) % 16 == 0) &&
-                (reinterpret_cast<uintptr_t>(w_out) % 16 == 0);
-  if (direct && !outputs_on_device) {
+  if (!outputs_on_device) {
     g_dev = static_cast<float*>(mapped_host(grad_out));
     w_dev = static_cast<float*>(mapped_host(w_out));
-    direct = (!grad_out || g_dev) && (!w_out || w_dev) && (reinterpret_cast<uintptr_t>(g_dev) % 16 == 0) &&
-             (reinterpret_cast<uintptr_t>(w_dev) % 16 == 0);
   }
-  if (direct) { dc.g_user = g_dev; dc.w_user = w_dev; }
+  const uintptr_t addr = reinterpret_cast<uintptr_t>(g_dev) | reinterpret_cast<uintptr_t>(w_dev);
+  const bool same = (ctx->K == 1 || ctx->ld == ctx->d) && addr % 16 == 0;
+  const bool direct = (!grad_out || g_dev) && (!w_out || w_dev) && (same || (ctx->K > 1 && addr % 4 == 0));
+  if (direct) {
+    dc.g_user = g_dev;
+    dc.w_user = w_dev;
+    dc.user_n = ctx->K == 1 ? ctx->d : ctx->P;
+    if (!same) {
+      dc.user_d = (int32_t)ctx->d;
+      dc.row4 = (uint32_t)(ctx->ld / 4);
+    }
+  }
   bool need_commit = true, need_decode = true;
   if (ctx->loss != PGC_SOFTMAX) {
     // K1 with its fused tail: commit (and, for small P, decode) in the same launch
@@ -1403,17 +1422,19 @@ int pgc_set_gc_encoding(pgc_ctx* ctx, const double* draws) {
   if (s > 0)
     PGC_CK(ctx, cudaMemcpyAsync(ctx->gc_draws, draws, (size_t)s * (n - 1) * sizeof(double), cudaMemcpyHostToDevice, st));
   PGC_CK(ctx, launch_gc_encoding(ctx->gc_draws, n, s, ctx->gc_coeff, ctx->status, st));
-  int h = 0;
-  PGC_CK(ctx, cudaMemcpyAsync(&h, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, st));
-  PGC_CK(ctx, cudaStreamSynchronize(st));
-  if (h == kErrSingular) {
+  const int rc = read_status(ctx);
+  if (rc == PGC_ESINGULAR && *ctx->status_h == kErrSingular) {
     // the draws leave some worker's system singular: keep the context usable
-    PGC_CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(int), st));
-    PGC_CK(ctx, cudaStreamSynchronize(st));
+    if (ctx->status != ctx->status_h) {
+      PGC_CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(int), st));
+      PGC_CK(ctx, cudaStreamSynchronize(st));
+    }
+    *ctx->status_h = 0;
+    ctx->broken = false;
     ctx->gc_ready = false;
     return PGC_ESINGULAR;
   }
-  if (h) return read_status(ctx);
+  if (rc) return rc;
   ctx->gc_ready = true;
   return PGC_OK;
 }

@@ -49,8 +49,11 @@ struct DecodeArgs {
   float lr;
   float* coeff_out;         // [n] per-worker coefficient a_i (written once per step)
   int* status;
-  float* g_user = nullptr;  // optional extra destinations of ghat and beta, same
-  float* w_user = nullptr;  // unpadded layout (used when ld == d)
+  float* g_user = nullptr;  // optional extra destinations of ghat and beta, unpadded:
+  float* w_user = nullptr;  // [K][d], on the device or in mapped host memory
+  int64_t user_n = 0;       // user_d == 0: their layout is [P]'s, cut off after user_n floats (16-byte aligned)
+  int32_t user_d = 0;       // != 0: their rows have user_d floats where [P]'s have 4 row4
+  uint32_t row4 = 1;
   int u_ready = 0;          // U[slot] already holds this step's slot total
   const float* pre = nullptr;  // with u_ready: the terms of the slots other than o_t, summed
                                // early (TcSoftmaxParams::pre_out)

@@ -46,6 +46,7 @@ constexpr int kTailMaxC = 4;   // slots per store on the fused tail's short rout
 // all threads of the CTA after its partials are written.  plan: shared
 // memory for the decode plan; gs_area / gs_bytes: idle shared memory for
 // the committed gradients of the short route; bar_flag: a shared int.
+template <int kUser>
 __device__ __forceinline__ void rows_fused_tail(const RowsArgs& a, DecodePlan& plan, uint8_t* gs_area,
                                                 int64_t gs_bytes, int* bar_flag) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -105,7 +106,7 @@ __device__ __forceinline__ void rows_fused_tail(const RowsArgs& a, DecodePlan& p
     __syncthreads();                   // this CTA's stores (and gs) are visible to all its threads
     if (blockIdx.x == 0 && warp == 0) write_coeffs_warp(a.dec, lane);
     if (!fast) {
-      decode_columns(a.dec, plan, q0, q1, (int)threadIdx.x, (int)blockDim.x);
+      decode_columns<kUser>(a.dec, plan, q0, q1, (int)threadIdx.x, (int)blockDim.x);
     } else if ((int64_t)threadIdx.x < nq) {
       // U[o_t] = sum over the evaluated partitions of their new gradients
       float4 un = f4zero();
@@ -122,7 +123,7 @@ __device__ __forceinline__ void rows_fused_tail(const RowsArgs& a, DecodePlan& p
         D = f4fma(plan.devc[q], Cr, D);
       }
       const float4 g = f4fma(plan.B, V, D);
-      store_outputs(dc, pq, g, f4fma(-dc.lr, g, wv));
+      store_outputs<kUser>(dc, pq, g, f4fma(-dc.lr, g, wv));
     }
     __syncthreads();
     // the last CTA out resets the counters for the next step

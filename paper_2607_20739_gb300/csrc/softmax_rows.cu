@@ -198,6 +198,7 @@ __host__ __device__ static RowsSmem rows_smem(int64_t ld, int nslots) {
 }
 static_assert(2 * kFw * kZp >= sizeof(DecodePlan), "the decode plan fits the partial-logit area");
 
+template <int kUser>
 __global__ void __launch_bounds__(kRThreads, 1)
 softmax_rows_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ RowsArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -583,7 +584,7 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     // ---- fused tail: commit, then decode + SGD (rows_tail.cuh); the decode
     // plan goes where the partial logits were, the committed gradients of
     // the short route where the slots were
-    rows_fused_tail(a, *reinterpret_cast<DecodePlan*>(zpart), sm, (int64_t)S * L.slot_bytes, &bar_flag);
+    rows_fused_tail<kUser>(a, *reinterpret_cast<DecodePlan*>(zpart), sm, (int64_t)S * L.slot_bytes, &bar_flag);
   }
   if (warp == 1) {
     // after a failure, wait (bounded) for the last commit before releasing TMEM
@@ -598,6 +599,8 @@ softmax_rows_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
+using RowsKernel = void (*)(const CUtensorMap, RowsArgs);
+
 int rows_slots(int64_t ld) {
   if (ld % (128 * kPairCtas) != 0 || ld > kRowsMaxLd) return 0;
   int s = kRowsMaxSlots;
@@ -636,13 +639,15 @@ static cudaLaunchConfig_t rows_config(int64_t ld, int nslots, int nctas, cudaLau
 
 int rows_max_ctas(int64_t ld, int nslots) {
   const size_t smem = rows_smem_bytes(ld, nslots);
-  if (cudaFuncSetAttribute(softmax_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return 0;
+  for (const RowsKernel k : {softmax_rows_kernel<kUserSame>, softmax_rows_kernel<kUserRows>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = rows_config(ld, nslots, kPairCtas, attr, false, 0);
-  int nc = 0;
-  if (cudaOccupancyMaxActiveClusters(&nc, softmax_rows_kernel, &cfg) != cudaSuccess) return 0;
+  int nc = 0, nc2 = 0;
+  if (cudaOccupancyMaxActiveClusters(&nc, softmax_rows_kernel<kUserSame>, &cfg) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&nc2, softmax_rows_kernel<kUserRows>, &cfg) != cudaSuccess)
+    return 0;
+  if (nc2 < nc) nc = nc2;
   return nc * kPairCtas;   // every pair co-resident (the fused tail's grid barriers need it)
 }
 
@@ -652,13 +657,14 @@ cudaError_t launch_softmax_rows(const void* tmX, const RowsArgs& a, int nctas, c
     return cudaErrorInvalidValue;
   if (a.box_blocks < 1 || (a.ld / kPairCtas / 64) % a.box_blocks != 0) return cudaErrorInvalidValue;
   const size_t smem = rows_smem_bytes(a.ld, a.nslots);
-  cudaError_t e = cudaFuncSetAttribute(softmax_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const RowsKernel kern = a.tail && a.dec.user_d ? softmax_rows_kernel<kUserRows> : softmax_rows_kernel<kUserSame>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = rows_config(a.ld, a.nslots, nctas, attr, a.pdl != 0, st);
   CUtensorMap x;
   std::memcpy(&x, tmX, sizeof(CUtensorMap));
-  return cudaLaunchKernelEx(&cfg, softmax_rows_kernel, x, a);
+  return cudaLaunchKernelEx(&cfg, kern, x, a);
 }
 
 }  // namespace pgc

@@ -154,11 +154,45 @@ __device__ __forceinline__ void store_split4(uint16_t* dst, int64_t stride, int6
   }
 }
 
+// The caller's copies of ghat and beta, written without the padding of the
+// parameter rows.  kUserSame: rows of ld = d floats, 16-byte aligned.
+// kUserPrefix: one class, the caller's array ends after user_n floats.
+// kUserRows: [K][user_d] behind rows of 4 row4 floats, any 4-byte alignment.
+enum { kUserSame = 0, kUserPrefix = 1, kUserRows = 2 };
+__device__ __forceinline__ void put4(float* dst, int n, float4 v) {
+  if (n >= 4 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+    *reinterpret_cast<float4*>(dst) = v;
+    return;
+  }
+  if (n > 0) dst[0] = v.x;
+  if (n > 1) dst[1] = v.y;
+  if (n > 2) dst[2] = v.z;
+  if (n > 3) dst[3] = v.w;
+}
+template <int kUser>
+__device__ __forceinline__ void store_user(const DecodeArgs& a, int64_t p, float4 g, float4 w) {
+  if constexpr (kUser == kUserSame) {
+    if (a.w_user) reinterpret_cast<float4*>(a.w_user)[p] = w;
+    if (a.g_user) reinterpret_cast<float4*>(a.g_user)[p] = g;
+  } else {
+    int64_t off = 4 * p, n = a.user_n - off;
+    if constexpr (kUser == kUserRows) {
+      const uint32_t k = (uint32_t)p / a.row4;                // P / 4 < 2^32: 4096 classes of 2^20 features
+      const int64_t j = 4 * (int64_t)((uint32_t)p - k * a.row4);
+      off = (int64_t)k * a.user_d + j;
+      n = a.user_d - j;
+    }
+    const int m = n < 4 ? (int)n : 4;
+    if (a.w_user) put4(a.w_user + off, m, w);
+    if (a.g_user) put4(a.g_user + off, m, g);
+  }
+}
+
+template <int kUser>
 __device__ __forceinline__ void store_outputs(const DecodeArgs& a, int64_t p, float4 g, float4 w) {
   reinterpret_cast<float4*>(a.w)[p] = w;
   reinterpret_cast<float4*>(a.gout)[p] = g;
-  if (a.w_user) reinterpret_cast<float4*>(a.w_user)[p] = w;
-  if (a.g_user) reinterpret_cast<float4*>(a.g_user)[p] = g;
+  store_user<kUser>(a, p, g, w);
   if (a.wb) {
     __nv_bfloat162 lo = __floats2bfloat162_rn(w.x, w.y);
     __nv_bfloat162 hi = __floats2bfloat162_rn(w.z, w.w);
@@ -169,24 +203,33 @@ __device__ __forceinline__ void store_outputs(const DecodeArgs& a, int64_t p, fl
   }
 }
 
-// store_outputs for the standalone decode kernels, which also serve the path
-// whose kernels read beta as three bf16 parts (the fused tails never do, and
-// the branch there cost the few-class kernel 2 us of its 57).
+// store_outputs for the standalone decode kernels, which serve every path:
+// beta as three bf16 parts, and the caller's arrays in any layout (the fused
+// tails are compiled for theirs: one more branch cost the few-class kernel 2 us
+// of its 57).
 __device__ __forceinline__ void store_outputs_any(const DecodeArgs& a, int64_t p, float4 g, float4 w) {
+  reinterpret_cast<float4*>(a.w)[p] = w;
+  reinterpret_cast<float4*>(a.gout)[p] = g;
+  if (a.g_user || a.w_user) {
+    if (a.user_d) store_user<kUserRows>(a, p, g, w);
+    else store_user<kUserPrefix>(a, p, g, w);
+  }
   if (a.wb_stride) {
     store_split4(a.wb, a.wb_stride, p, w);
-    reinterpret_cast<float4*>(a.w)[p] = w;
-    reinterpret_cast<float4*>(a.gout)[p] = g;
-    if (a.w_user) reinterpret_cast<float4*>(a.w_user)[p] = w;
-    if (a.g_user) reinterpret_cast<float4*>(a.g_user)[p] = g;
-  } else {
-    store_outputs(a, p, g, w);
+  } else if (a.wb) {
+    __nv_bfloat162 lo = __floats2bfloat162_rn(w.x, w.y);
+    __nv_bfloat162 hi = __floats2bfloat162_rn(w.z, w.w);
+    uint2 pk;
+    pk.x = *reinterpret_cast<uint32_t*>(&lo);
+    pk.y = *reinterpret_cast<uint32_t*>(&hi);
+    reinterpret_cast<uint2*>(a.wb)[p] = pk;
   }
 }
 
 // Decode + SGD of the float4 columns [q0, q1), every column handled by one
 // thread (tid of nthr) and no barriers.  When the counts fit the unrolled
 // bounds all loads of a column are issued back to back; otherwise plain loops.
+template <int kUser>
 __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const DecodePlan& pl, int64_t q0, int64_t q1,
                                                int tid, int nthr) {
   constexpr int kMaxO = 8, kMaxC = 4, kMaxD = 4;
@@ -245,7 +288,7 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
     const float4 g = f4fma(B, V, D);
     float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
-    store_outputs(a, p, g, w);
+    store_outputs<kUser>(a, p, g, w);
   }
 }
 
