@@ -127,8 +127,8 @@ struct pgc_ctx {
   double* loss_blocks = nullptr;
   double* loss_out = nullptr;
   int64_t* loss_desc = nullptr;
-  int* counters = nullptr;   // [n + 3]: per-partition arrivals, committed partitions,
-                             // work-item counter, finished producers (zero between steps)
+  int* counters = nullptr;   // [n + 4]: per-partition arrivals, committed partitions, work-item
+                             // counter, finished producers, loss blocks (zero between steps)
   bool pdl = true;           // chain the step's kernels with programmatic dependent launch
   int tail_mode = 0;         // fused tail of the gradient kernel (see GradRowsArgs)
   int mode = PGC_MODE_PGC;   // training scheme (PGC_MODE_*)
@@ -179,6 +179,8 @@ struct pgc_ctx {
   int lw_nc = 0;               // softmax loss on the tensor cores: its clusters (0: tiled CUDA-core logits)
   int lw_Kp = 0, lw_ncb = 0;   // its class blocks: ncb of Kp
   uint16_t* lw = nullptr;      // W parts [ncb][3][Kp][ld] (split path: wb)
+  float2* row_stats = nullptr; // its (max, sum of exp) [ncb][rows], then
+  float* row_lab = nullptr;    // the label logits [rows]
   void* tmXl = nullptr;        // device tensor map of X over all rows
   alignas(64) unsigned char tmWl[128];   // W parts
   double* loss_h = nullptr;    // pinned host copy of the loss
@@ -574,7 +576,7 @@ void free_all(pgc_ctx* ctx) {
   ctx->ev_pool.clear();
   void* ptrs[] = {ctx->X, ctx->y, ctx->w, ctx->wb, ctx->store, ctx->U, ctx->gout, ctx->partials, ctx->Z,
                   ctx->coeff, ctx->status == ctx->status_h ? nullptr : ctx->status, ctx->loss_blocks, ctx->loss_out, ctx->tables, ctx->counters, ctx->Rb,
-                  ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre, ctx->R3, ctx->tmX, ctx->tmXl,
+                  ctx->gc_coeff, ctx->gc_d, ctx->gc_draws, ctx->gc_wts, ctx->pre, ctx->R3, ctx->tmX, ctx->tmXl, ctx->row_stats,
                   ctx->lw == ctx->wb ? nullptr : ctx->lw};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -873,19 +875,19 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   for (auto& ph : ctx->phases) max_zpad = std::max(max_zpad, ph.zpad_total);
   if (loss == PGC_SOFTMAX && !no_split && ctx->total_rows < (int64_t(1) << 31) - kSplitRows) {
     // the loss on the tensor cores, if the parts of W fit
-    ctx->lw_nc = split_max_clusters(kSplitLoss, dtype, std::min(K, kSplitMaxClasses));
+    const int nc = split_max_clusters(kSplitLoss, dtype, std::min(K, kSplitMaxClasses));
     ctx->lw_Kp = split_kp(std::min(K, kSplitMaxClasses));
     ctx->lw_ncb = (int)((K + ctx->lw_Kp - 1) / ctx->lw_Kp);
+    const size_t parts = (size_t)3 * ctx->lw_ncb * ctx->lw_Kp * ctx->ld * 2;
+    const size_t rows_b = (size_t)ctx->total_rows * (ctx->lw_ncb * sizeof(float2) + sizeof(float));
     if (ctx->split) ctx->lw = ctx->wb;
-    else if (ctx->lw_nc > 0 &&
-             cudaMalloc((void**)&ctx->lw, (size_t)3 * ctx->lw_ncb * ctx->lw_Kp * ctx->ld * 2) != cudaSuccess) {
-      cudaGetLastError();
-      ctx->lw = nullptr;
-      ctx->lw_nc = 0;
-    }
-    if (ctx->lw_nc > 0) {
+    if (nc > 0 && (ctx->split || cudaMalloc((void**)&ctx->lw, parts) == cudaSuccess) &&
+        cudaMalloc((void**)&ctx->row_stats, rows_b) == cudaSuccess) {
+      ctx->lw_nc = nc;
+      ctx->row_lab = reinterpret_cast<float*>(ctx->row_stats + ctx->total_rows * ctx->lw_ncb);
       PGC_ALLOC(ctx->tmXl, 128);
-      ctx->loss_nblocks = 8 * ctx->lw_nc;
+    } else {
+      cudaGetLastError();
     }
   } else if (loss != PGC_SOFTMAX) {
     ctx->loss_nblocks = 8 * ctx->sm_count;
@@ -939,7 +941,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   PGC_ALLOC(ctx->loss_blocks, (size_t)ctx->loss_nblocks * sizeof(double));
   PGC_ALLOC(ctx->loss_out, sizeof(double));
   PGC_ALLOC(ctx->tables, tab.size());
-  PGC_ALLOC(ctx->counters, (size_t)(n + 3) * sizeof(int));
+  PGC_ALLOC(ctx->counters, (size_t)(n + 4) * sizeof(int));
   if (gc_weighted) {
     PGC_ALLOC(ctx->gc_coeff, (size_t)n * ctx->c * sizeof(double));
     PGC_ALLOC(ctx->gc_d, (size_t)(n + 2) * sizeof(double));
@@ -956,7 +958,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->gout, 0, Pb, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->coeff, 0, (size_t)n * sizeof(float), st);
   if (e == cudaSuccess && ctx->status != ctx->status_h) e = cudaMemsetAsync(ctx->status, 0, sizeof(int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->counters, 0, (size_t)(n + 3) * sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->counters, 0, (size_t)(n + 4) * sizeof(int), st);
   if (e == cudaSuccess && gc_weighted) e = cudaMemsetAsync(ctx->gc_wts, 0, (size_t)n * ctx->c * sizeof(float), st);
   if (e == cudaSuccess && gc_weighted) e = cudaMemsetAsync(ctx->gc_d, 0, (size_t)(n + 2) * sizeof(double), st);
   if (e == cudaSuccess && w0)
@@ -1355,12 +1357,13 @@ int pgc_loss(pgc_ctx* ctx, double* loss_out) {
     if (ctx->lw != ctx->wb) PGC_CK(ctx, launch_split_weights(ctx->w, ctx->lw, ctx->K, ctx->ld, ctx->lw_Kp, ctx->stream));
     SplitArgs a = {};
     a.K = (int)ctx->K; a.Kp = ctx->lw_Kp; a.ncb = ctx->lw_ncb; a.ld = ctx->ld; a.nkb = (int)(ctx->ld / 64);
-    a.chunk = kSplitChunk; a.tmX = ctx->tmXl; a.rows = ctx->total_rows; a.blocksum = ctx->loss_blocks;
-    a.nunits = (int)((ctx->total_rows + kSplitRows - 1) / kSplitRows);
+    a.chunk = kSplitChunk; a.tmX = ctx->tmXl; a.rows = ctx->total_rows;
+    a.row_stats = ctx->row_stats; a.row_lab = ctx->row_lab;
+    a.nunits = ctx->lw_ncb * (int)((ctx->total_rows + kSplitRows - 1) / kSplitRows);
     a.y = static_cast<const int32_t*>(ctx->y); a.status = ctx->status;
-    PGC_CK(ctx, launch_split(kSplitLoss, ctx->dtype, ctx->tmWl, a, ctx->lw_nc, false, ctx->stream));
-    PGC_CK(ctx, launch_loss_finish(ctx->loss_blocks, 8 * std::min(a.nunits, ctx->lw_nc), ctx->total_rows, ctx->loss_out,
-                                   ctx->stream));
+    PGC_CK(ctx, launch_split(kSplitLoss, ctx->dtype, ctx->tmWl, a, ctx->lw_nc, ctx->pdl, ctx->stream));
+    PGC_CK(ctx, launch_loss_combine(ctx->row_stats, ctx->row_lab, ctx->total_rows, ctx->lw_ncb, ctx->loss_blocks,
+                                    ctx->loss_nblocks, ctx->counters + ctx->n + 3, ctx->loss_out, ctx->stream));
   } else {
     LossArgs a;
     a.loss = ctx->loss; a.dtype = ctx->dtype; a.ld = ctx->ld; a.K = ctx->K; a.rows = ctx->total_rows;

@@ -185,8 +185,6 @@ struct LossArgs {
   const int64_t* chunk_desc; // device [3 * nchunks]: {row0, rows, 0} per chunk
 };
 cudaError_t launch_loss(const LossArgs& a, cudaStream_t st);
-// out = (sum of blocksum) / rows
-cudaError_t launch_loss_finish(const double* blocksum, int nblocks, int64_t rows, double* out, cudaStream_t st);
 
 // ---- tensor-core logits GEMM (tc_gemm.cu) --------------------------------
 // Z[r][k] = sum_j X[r][j] Wb[k][j] (A = X K-major, B = Wb K-major), for the
@@ -406,11 +404,12 @@ struct SplitArgs {
   int ndest;
   float* store;
   int* status;
-  // loss: row tiles nunits = ceil(rows / 256) of one map over all rows, ncb
-  // blocks of Kp classes; per epilogue warp of every CTA one sum of log sum exp - z_y
+  // loss: nunits = ncb x ceil(rows / 256) units over all rows (one map), class
+  // block n % ncb of row tile n / ncb; (max, sum of exp) per block and row, label logits
   int64_t rows;
   int ncb;
-  double* blocksum;         // [4 x CTAs]
+  float2* row_stats;        // [ncb][rows]
+  float* row_lab;           // [rows]
 };
 // Clusters of two CTAs that fit at once (0: cannot launch).
 int split_max_clusters(int mode, int dtype, int64_t K);
@@ -420,6 +419,9 @@ int split_max_clusters(int mode, int dtype, int64_t K);
 // kSplitLoss: tmB = W parts [ncb][3 Kp][ld]; tmX: one map over all rows, box as kSplitLogits.
 cudaError_t launch_split(int mode, int dtype, const void* tmB, const SplitArgs& a, int nclusters, bool pdl,
                          cudaStream_t st);
+// out = mean over the rows of log sum exp - label logit; ticket: a zero word, returned to zero
+cudaError_t launch_loss_combine(const float2* stats, const float* lab, int64_t rows, int ncb, double* blocksum,
+                                int max_blocks, int* ticket, double* out, cudaStream_t st);
 // w [K][ld] -> parts [ceil(K / Kp)][3][Kp][ld] (rows past K are not written)
 cudaError_t launch_split_weights(const float* src, uint16_t* dst, int64_t K, int64_t ld, int Kp, cudaStream_t st);
 // 2-D tensor map [outer][inner], row pitch in bytes, box {box_inner, box_outer}, 128-byte swizzle or none

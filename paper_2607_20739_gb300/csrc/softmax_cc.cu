@@ -363,11 +363,6 @@ __global__ void loss_finish(const double* blocksum, int nblocks, int64_t rows, d
   if (threadIdx.x == 0) *out = s / (double)rows;
 }
 
-cudaError_t launch_loss_finish(const double* blocksum, int nblocks, int64_t rows, double* out, cudaStream_t st) {
-  loss_finish<<<1, 32, 0, st>>>(blocksum, nblocks, rows, out);
-  return cudaGetLastError();
-}
-
 __global__ void zero_doubles(double* p, int n) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0.0;
 }
@@ -397,7 +392,8 @@ cudaError_t launch_loss(const LossArgs& a, cudaStream_t st) {
       if (e != cudaSuccess) return e;
     }
   }
-  return launch_loss_finish(a.blocksum, a.nblocks, a.rows, a.out, st);
+  loss_finish<<<1, 32, 0, st>>>(a.blocksum, a.nblocks, a.rows, a.out);
+  return cudaGetLastError();
 }
 
 }  // namespace pgc

@@ -44,11 +44,14 @@
 // thread) into the partition's partial or, if one unit holds the whole
 // partition, times 1/m_e straight into the stores.
 //
-// The same logits with a third epilogue give the loss F (any K): class blocks
-// of up to 128 in turn per row tile, X read again (from L2) for each, every
-// row's log sum exp kept in its thread.  Before, the tiled CUDA-core logits
+// The same logits with a third epilogue give the loss F (any K): a unit is a
+// row tile and a block of up to 128 classes (X comes from L2 for all but one of a
+// tile's blocks); every row's max and sum of exp per block go to memory and a
+// small kernel combines them.  Before, the tiled CUDA-core logits
 // went through memory, and one more kernel reduced them: a step with its loss on
-// 8 partitions of about 600 x 1500 bf16, 300 classes, took 473 us, now 202.
+// 8 partitions of about 600 x 1500 bf16, 300 classes, took 473 us; now 144
+// (184 with the class blocks of a tile one after the other in one cluster: 20
+// of 76 clusters busy).
 //
 // Every wait is bounded; on a failure the kernel flags the status word, all
 // roles wind down, and TMEM is released after the MMAs issued so far.
@@ -215,16 +218,12 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
   grid_dep_wait();                       // W (R) is the previous kernel's output
 
   const int ncl = (int)gridDim.x >> 1, cid = (int)blockIdx.x >> 1;
-  // loss: every class block of a row tile in turn
-  const int ncb = kMode == kSplitLoss ? p.ncb : 1;
-  const int my_units = p.nunits > cid ? (p.nunits - cid + ncl - 1) / ncl * ncb : 0;
+  // loss: unit = class block e of a row tile, the blocks of a tile side by side
+  const int my_units = p.nunits > cid ? (p.nunits - cid + ncl - 1) / ncl : 0;
   auto unit = [&](int i) {
-    if constexpr (kMode == kSplitLoss) {
-      const int tile = cid + i / ncb * ncl;
-      return SplitUnit{i % ncb, 0, 0, tile * kSplitRows, (int)p.rows, 0, 0, 0};   // e: class block
-    } else {
-      return p.units[cid + i * ncl];
-    }
+    const int n = cid + i * ncl;
+    if constexpr (kMode == kSplitLoss) return SplitUnit{n % p.ncb, 0, 0, n / p.ncb * kSplitRows, (int)p.rows, 0, 0, 0};
+    else return p.units[n];
   };
   auto blocks_of = [&](const SplitUnit& u) { return kGrad ? (u.rows + kSK - 1) / kSK : p.nkb; };
 
@@ -393,8 +392,6 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
     const int q = warp & 3, t = q * 32 + lane;               // row (logits) or feature (gradient) of the CTA's 128
     int tt = 0;
     bool ok = true;
-    double loss = 0.0;                                       // loss: this thread's rows so far,
-    float run_m = 0.f, run_s = 0.f, z_lab = 0.f;             // its row's max, sum of exp and label logit
     for (int i = 0; i < my_units && ok; ++i) {
       const SplitUnit u = unit(i);
       const int nkb = blocks_of(u), nchunk = (nkb + p.chunk - 1) / p.chunk;
@@ -438,25 +435,23 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
         if (lane == 0) mbar_arrive(&corr_empty[cor]);
       }
       if constexpr (kMode == kSplitLoss) {
-        // log sum_k exp(z_k) - z_y over the class blocks of this thread's row
+        // this thread's row: max and sum of exp over the class block, the label's
+        // logit if it is one of them
         const int row = u.r0 + rank * kSM + t;
-        const bool valid = row < u.rows;
-        const int c0 = u.e * Kp, nc = p.K - c0 < Kp ? p.K - c0 : Kp;
-        const int lab = valid ? p.y[row] - c0 : -1;
-        if (u.e == 0) { run_m = -INFINITY; run_s = 0.f; z_lab = 0.f; }
-        float m = run_m;
+        if (row < u.rows) {
+          const int c0 = u.e * Kp, nc = p.K - c0 < Kp ? p.K - c0 : Kp;
+          const int lab = p.y[row] - c0;
+          float m = -INFINITY, sum = 0.f;
 #pragma unroll
-        for (int c = 0; c < NCH * 32; ++c) {
-          if (c < nc) m = fmaxf(m, z[c]);
-          if (c < nc && c == lab) z_lab = z[c];
+          for (int c = 0; c < NCH * 32; ++c) {
+            if (c < nc) m = fmaxf(m, z[c]);
+            if (c < nc && c == lab) p.row_lab[row] = z[c];
+          }
+#pragma unroll
+          for (int c = 0; c < NCH * 32; ++c)
+            if (c < nc) sum += expf(z[c] - m);
+          p.row_stats[(int64_t)u.e * p.rows + row] = make_float2(m, sum);
         }
-        float sum = run_s == 0.f ? 0.f : run_s * expf(run_m - m);
-#pragma unroll
-        for (int c = 0; c < NCH * 32; ++c)
-          if (c < nc) sum += expf(z[c] - m);
-        run_m = m;
-        run_s = sum;
-        if (u.e == ncb - 1 && valid) loss += (double)m + log((double)sum) - (double)z_lab;
       } else if constexpr (!kGrad) {
         // R = softmax(Z) - onehot(y) of this thread's row, zero past the partition
         const int row = u.r0 + rank * kSM + t;
@@ -515,11 +510,6 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
           }
         }
       }
-    }
-    if constexpr (kMode == kSplitLoss) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-      if (lane == 0) p.blocksum[blockIdx.x * 4 + (warp - 2)] = loss;
     }
   }
   __syncthreads();
@@ -609,6 +599,66 @@ cudaError_t launch_split(int mode, int dtype, const void* tmB, const SplitArgs& 
   CUtensorMap b;
   std::memcpy(&b, tmB, sizeof(CUtensorMap));
   return cudaLaunchKernelEx(&cfg, k, b, a);
+}
+
+// Sum over the rows of log sum_k exp(z_k) - z_y from the class blocks' (max, sum
+// of exp) and the label's logit; the last block to finish adds the blocks'
+// sums in order and divides by the rows (ticket returns to 0).
+__global__ void __launch_bounds__(256) loss_combine_kernel(const float2* __restrict__ stats, const float* __restrict__ lab,
+                                                           int64_t rows, int ncb, double* blocksum, int* ticket,
+                                                           double* out) {
+  __shared__ double red[8];
+  __shared__ int last;
+  grid_dep_wait();
+  double acc = 0.0;
+  for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < rows; r += (int64_t)gridDim.x * 256) {
+    float M = -INFINITY;
+    for (int b = 0; b < ncb; ++b) M = fmaxf(M, stats[b * rows + r].x);
+    float s = 0.f;
+    for (int b = 0; b < ncb; ++b) {
+      const float2 v = stats[b * rows + r];
+      s += v.y * expf(v.x - M);
+    }
+    acc += (double)M + log((double)s) - (double)lab[r];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < 8; ++i) t += red[i];
+    blocksum[blockIdx.x] = t;
+    last = atomic_add_acq_rel(ticket, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last && threadIdx.x < 32) {
+    __threadfence();
+    double t = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) t += __ldcg(blocksum + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) {
+      *out = t / (double)rows;
+      *ticket = 0;
+    }
+  }
+}
+
+cudaError_t launch_loss_combine(const float2* stats, const float* lab, int64_t rows, int ncb, double* blocksum,
+                                int max_blocks, int* ticket, double* out, cudaStream_t st) {
+  int64_t blocks = (rows + 255) / 256;
+  if (blocks > max_blocks) blocks = max_blocks;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, loss_combine_kernel, stats, lab, rows, ncb, blocksum, ticket, out);
 }
 
 // fp32 [K][ld] -> bf16 parts [K / Kp blocks][3][Kp][ld] (Kp classes per block)
