@@ -45,25 +45,25 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
 }
 
 // Solve the rows x cols system M[:, 0:cols] x = M[:, cols] (row-major, leading
-// dimension kGcLd, rows >= cols, rows <= 64) in place by one warp: lane l owns
+// dimension ld, rows >= cols, rows <= 64) in place by one warp: lane l owns
 // rows l and l + 32.  Pivot rows are chosen per column by largest magnitude
 // among the rows not used yet (no rows move; piv[] records the order); rows
 // left over after cols pivots are not used (the caller checks consistency).
 // Writes x[0:cols] (shared) and returns false on a singular pivot.
-__device__ bool warp_solve(double* M, int rows, int cols, double* x, int* piv) {
+__device__ bool warp_solve(double* M, int ld, int rows, int cols, double* x, int* piv) {
   const int lane = threadIdx.x & 31;
   bool used0 = lane >= rows, used1 = lane + 32 >= rows;
   double scale = 0.0;
   for (int r = lane; r < rows; r += 32)
-    for (int q = 0; q < cols; ++q) scale = fmax(scale, fabs(M[r * kGcLd + q]));
+    for (int q = 0; q < cols; ++q) scale = fmax(scale, fabs(M[r * ld + q]));
   scale = warp_max_f64(scale);
   for (int k = 0; k < cols; ++k) {
     // pivot: the unused row with the largest |M[r][k]|; ties to the lower row
     double bv = -1.0;
     int br = rows;
-    if (!used0) { bv = fabs(M[lane * kGcLd + k]); br = lane; }
+    if (!used0) { bv = fabs(M[lane * ld + k]); br = lane; }
     if (!used1) {
-      const double v = fabs(M[(lane + 32) * kGcLd + k]);
+      const double v = fabs(M[(lane + 32) * ld + k]);
       if (v > bv) { bv = v; br = lane + 32; }
     }
 #pragma unroll
@@ -78,12 +78,12 @@ __device__ bool warp_solve(double* M, int rows, int cols, double* x, int* piv) {
     if (p == lane) used0 = true;
     if (p == lane + 32) used1 = true;
     __syncwarp();
-    const double* Mp = M + p * kGcLd;
+    const double* Mp = M + p * ld;
     const double inv = 1.0 / Mp[k];
     for (int h = 0; h < 2; ++h) {
       const int r = lane + 32 * h;
       if (h == 0 ? used0 : used1) continue;
-      double* Mr = M + r * kGcLd;
+      double* Mr = M + r * ld;
       const double f = Mr[k] * inv;
       for (int q = k + 1; q <= cols; ++q) Mr[q] = fma(-f, Mp[q], Mr[q]);
       Mr[k] = 0.0;
@@ -92,7 +92,7 @@ __device__ bool warp_solve(double* M, int rows, int cols, double* x, int* piv) {
   }
   // back-substitution in pivot order; lanes split the inner sum
   for (int k = cols - 1; k >= 0; --k) {
-    const double* Mp = M + piv[k] * kGcLd;
+    const double* Mp = M + piv[k] * ld;
     double acc = 0.0;
     for (int q = k + 1 + lane; q < cols; q += 32) acc = fma(Mp[q], x[q], acc);
     acc = warp_sum_f64(acc);
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(32) gc_encoding_kernel(const double* __restric
     M[r * kGcLd + s] = -h_entry(draws, n, r, j, rowsum);
   }
   __syncwarp();
-  const bool ok = s == 0 || warp_solve(M, s, s, x, piv);
+  const bool ok = s == 0 || warp_solve(M, kGcLd, s, s, x, piv);
   if (!ok) {
     if (lane == 0) atomicOr(status, kErrSingular);
     return;
@@ -141,13 +141,21 @@ __global__ void __launch_bounds__(32) gc_encoding_kernel(const double* __restric
 // grid 1, block 32.  Outputs: d [n] (0 for stragglers), wts [n][c] fp32
 // d_j c_{j,l} / n, coeff_out [n] fp32 d_j / n (the per-worker coefficient of
 // the coded gradient), alpha [2] = max, min of d_j c_{j,l} over received j.
+// The solve needs only the mask and the encoding: launched as a dependent of
+// the gradient kernel, with shared memory for this n alone (6 KB at n = 24), it
+// runs beside it on an SM the gradient kernel also uses, and only its outputs
+// wait for that kernel (the previous step's decode may still read the old
+// ones).  naive_cr, 8 x 8192 x 1024: 70.0 us per step with the solve after it, 50.8
+// beside it (the gradient kernel takes 47).
 __global__ void __launch_bounds__(32) gc_weights_kernel(GcWeightsArgs a) {
-  __shared__ double M[kGcMaxN * kGcLd];
-  __shared__ double x[kGcMaxN];
-  __shared__ int piv[kGcMaxN];
-  __shared__ int recv[kGcMaxN];
+  extern __shared__ double gc_smem[];
   const int lane = threadIdx.x;
-  const int n = a.n, c = a.c;
+  const int n = a.n, c = a.c, ld = n + 1;
+  double* M = gc_smem;                       // [n][ld]
+  double* x = M + n * ld;                    // [n]
+  int* piv = reinterpret_cast<int*>(x + n);  // [n]
+  int* recv = piv + n;                       // [n]
+  grid_dep_launch();
   // the received workers, ascending
   int nr = 0;
   for (int base = 0; base < n; base += 32) {
@@ -159,6 +167,7 @@ __global__ void __launch_bounds__(32) gc_weights_kernel(GcWeightsArgs a) {
   }
   __syncwarp();
   if (nr != n - a.s) {
+    grid_dep_wait();
     for (int q = lane; q < n * c; q += 32) a.wts[q] = 0.f;
     if (lane == 0) atomicOr(a.status, kErrBadMask);
     return;
@@ -167,12 +176,12 @@ __global__ void __launch_bounds__(32) gc_weights_kernel(GcWeightsArgs a) {
   for (int k = lane; k < n; k += 32) {
     for (int m = 0; m < nr; ++m) {
       const int l = (k - recv[m] + n) % n;
-      M[k * kGcLd + m] = l < c ? a.coeff[(int64_t)recv[m] * c + l] : 0.0;
+      M[k * ld + m] = l < c ? a.coeff[(int64_t)recv[m] * c + l] : 0.0;
     }
-    M[k * kGcLd + nr] = 1.0;
+    M[k * ld + nr] = 1.0;
   }
   __syncwarp();
-  bool ok = warp_solve(M, n, nr, x, piv);
+  bool ok = warp_solve(M, ld, n, nr, x, piv);
   // consistency: every partition's decoding coefficients must sum to 1
   if (ok) {
     double res = 0.0, xmax = 0.0, bmax = 0.0;
@@ -194,6 +203,7 @@ __global__ void __launch_bounds__(32) gc_weights_kernel(GcWeightsArgs a) {
     bmax = warp_max_f64(bmax);
     ok = res <= kGcResidTol * (1.0 + xmax * bmax);
   }
+  grid_dep_wait();
   if (!ok) {
     // no weights: the decode leaves beta unchanged and the host reports the error
     for (int q = lane; q < n * c; q += 32) a.wts[q] = 0.f;
@@ -230,14 +240,14 @@ __global__ void __launch_bounds__(32) gc_weights_kernel(GcWeightsArgs a) {
 
 // One float4 column per thread, grid-stride; the received (worker, slot)
 // weights are compacted into shared memory in (worker, slot) order and each
-// column's sum issues eight loads at a time.
+// column's sum issues sixteen loads at a time.
 __global__ void __launch_bounds__(256) gc_decode_kernel(DecodeArgs a, const float* __restrict__ wts) {
-  __shared__ int qi[kGcMaxN * kGcMaxN];
-  __shared__ float qw[kGcMaxN * kGcMaxN];
+  extern __shared__ int qi[];                // [n c], then the weights [n c]
   __shared__ int qn;
+  const int nw = a.n * a.c;
+  float* qw = reinterpret_cast<float*>(qi + nw);
   grid_dep_launch();
   grid_dep_wait();
-  const int nw = a.n * a.c;
   if (threadIdx.x < 32) {
     int cnt = 0;
     for (int base = 0; base < nw; base += 32) {
@@ -260,12 +270,12 @@ __global__ void __launch_bounds__(256) gc_decode_kernel(DecodeArgs a, const floa
   const float4* store = reinterpret_cast<const float4*>(a.store);
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P4; p += (int64_t)gridDim.x * blockDim.x) {
     float4 g = f4zero();
-    for (int j0 = 0; j0 < cnt; j0 += 8) {
-      float4 v[8];
+    for (int j0 = 0; j0 < cnt; j0 += 16) {
+      float4 v[16];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = j0 + u < cnt ? __ldcg(store + (int64_t)qi[j0 + u] * P4 + p) : f4zero();
+      for (int u = 0; u < 16; ++u) v[u] = j0 + u < cnt ? __ldcg(store + (int64_t)qi[j0 + u] * P4 + p) : f4zero();
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
+      for (int u = 0; u < 16; ++u)
         if (j0 + u < cnt) g = f4fma(qw[j0 + u], v[u], g);
     }
     float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
@@ -282,21 +292,24 @@ cudaError_t launch_gc_encoding(const double* draws, int n, int s, double* coeff,
 
 cudaError_t launch_gc_decode(const GcWeightsArgs& w, const DecodeArgs& a, cudaStream_t st, bool pdl, int sm_count) {
   if (a.n < 1 || a.n > kGcMaxN || a.c < 1 || a.c > a.n) return cudaErrorInvalidValue;
-  gc_weights_kernel<<<1, 32, 0, st>>>(w);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  int64_t blocks = (a.P / 4 + 255) / 256;
-  if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
-  if (blocks < 1) blocks = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3(256);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(32);
+  cfg.dynamicSmemBytes = (size_t)a.n * (a.n + 2) * sizeof(double) + 2 * (size_t)a.n * sizeof(int);   // at most 35 KB
+  cudaError_t e = cudaLaunchKernelEx(&cfg, gc_weights_kernel, w);
+  if (e != cudaSuccess) return e;
+  int64_t blocks = (a.P / 4 + 255) / 256;
+  if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
+  if (blocks < 1) blocks = 1;
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = (size_t)a.n * a.c * (sizeof(int) + sizeof(float));   // at most 32 KB
   return cudaLaunchKernelEx(&cfg, gc_decode_kernel, a, static_cast<const float*>(w.wts));
 }
 
