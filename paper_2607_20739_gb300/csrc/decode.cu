@@ -3,6 +3,7 @@
 //   K4 commit_kernel  one CTA column-slice per evaluated partition: the new
 //                     gradient g_e = (1/m_e) * ordered sum of its partials,
 //                     written into every store that keeps the copy (§VI-A).
+//                     Below 2^20 parameters the decode kernel does it first.
 //   K6 decode_kernel  decode coefficients derived on the device from the
 //                     straggler mask (§IV-A, §V-B), decode, SGD (§III).
 // Both may be launched as programmatic dependents of the previous kernel:
@@ -70,16 +71,48 @@ cudaError_t launch_commit(const CommitArgs& a, cudaStream_t st, bool pdl) {
   return launch_maybe_pdl(pdl, commit_slice_kernel, dim3((unsigned)bx, (unsigned)a.nE), dim3(threads), st, a, slice4);
 }
 
-__global__ void __launch_bounds__(kDecX * kDecY) decode_kernel(DecodeArgs a) {
+// kCommit: the step's commit first, for the same columns (a column's decode
+// reads only that column of the stores, so a CTA barrier is enough): thread
+// row y sums the items of partitions y, y + kDecY, ..., in item order.  One
+// launch instead of two.
+template <bool kCommit>
+__global__ void __launch_bounds__(kDecX * kDecY) decode_kernel(DecodeArgs a, CommitArgs cm) {
   __shared__ DecodePlan pl;
-  __shared__ float4 red[kDecY][kDecX];
+  __shared__ float4 red[2 * kDecY][kDecX];
   grid_dep_launch();
   if (threadIdx.x < 32) derive_plan_warp(a, pl, threadIdx.x);   // needs only the mask
   __syncthreads();
   grid_dep_wait();
   if (blockIdx.x == 0 && threadIdx.x < 32) write_coeffs_warp(a, threadIdx.x);
+  const int64_t P4 = a.P / 4, nq = (P4 + kDecX - 1) / kDecX;
   auto bar = [] { __syncthreads(); };
-  decode_chunks(a, pl, red, (int)threadIdx.x, blockIdx.x, gridDim.x, bar);
+  for (int64_t q = blockIdx.x; q < nq; q += gridDim.x) {
+    if constexpr (kCommit) {
+      const int64_t p = q * kDecX + threadIdx.x % kDecX;
+      if (p < P4) {
+        const float4* src = reinterpret_cast<const float4*>(cm.partials) + p;
+        for (int e = threadIdx.x / kDecX; e < cm.nE; e += kDecY) {
+          const int i0 = cm.e_item0[e], i1 = cm.e_item0[e + 1];
+          float4 acc = f4zero();
+          for (int it = i0; it < i1; it += 8) {
+            float4 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = it + u < i1 ? __ldcg(src + (int64_t)(it + u) * P4) : f4zero();
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc = f4add(acc, v[u]);
+          }
+          const float sc = cm.e_scale[e];
+          acc = make_float4(acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc);
+          for (int k = 0; k < cm.ndest; ++k) {
+            const int dst = cm.e_dest[(int64_t)e * cm.ndest + k];
+            if (dst >= 0) reinterpret_cast<float4*>(cm.store)[(int64_t)dst * P4 + p] = acc;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    decode_chunk(a, pl, red, (int)threadIdx.x, q, bar);
+  }
 }
 
 // Sum of cnt float4 loads base[off(j)], j = 0..cnt-1, issued eight at a time
@@ -98,7 +131,7 @@ __device__ __forceinline__ float4 sum_loads8(const float4* base, int cnt, Off of
 }
 
 // Decode + SGD for large P: one thread per float4 column, grid-stride, no
-// barriers after the plan.  Same arithmetic as decode_chunks.
+// barriers after the plan.  Same arithmetic as decode_chunk.
 __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
   __shared__ DecodePlan pl;
   grid_dep_launch();
@@ -166,9 +199,12 @@ __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
 // Columns from which the one-thread-per-column decode is used.
 constexpr int64_t kWideDecodeMinP4 = 1 << 18;
 
-cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st, bool pdl, int sm_count) {
+bool decode_commits(int64_t P) { return P / 4 < kWideDecodeMinP4; }
+
+cudaError_t launch_decode(const DecodeArgs& a, const CommitArgs* cm, cudaStream_t st, bool pdl, int sm_count) {
   if (a.n > kMaxWorkers || a.owners > kMaxWorkers) return cudaErrorInvalidValue;
   if (a.P / 4 >= kWideDecodeMinP4) {
+    if (cm) return cudaErrorInvalidValue;
     int64_t blocks = (a.P / 4 + 255) / 256;
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     return launch_maybe_pdl(pdl, decode_wide_kernel, dim3((unsigned)blocks), dim3(256), st, a);
@@ -177,7 +213,8 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st, bool pdl, int sm
   int64_t chunks = (P4 + kDecX - 1) / kDecX;
   int64_t blocks = chunks < (int64_t)sm_count * 8 ? chunks : (int64_t)sm_count * 8;
   if (blocks < 1) blocks = 1;
-  return launch_maybe_pdl(pdl, decode_kernel, dim3((unsigned)blocks), dim3(kDecX * kDecY), st, a);
+  if (cm) return launch_maybe_pdl(pdl, decode_kernel<true>, dim3((unsigned)blocks), dim3(kDecX * kDecY), st, a, *cm);
+  return launch_maybe_pdl(pdl, decode_kernel<false>, dim3((unsigned)blocks), dim3(kDecX * kDecY), st, a, CommitArgs{});
 }
 
 // ---------------------------------------------------------------------------

@@ -1293,13 +1293,16 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
     PGC_CK(ctx, record_event(ctx));
   }
   PGC_CK(ctx, record_event(ctx));
+  CommitArgs cm = {};
+  const bool commit_in_decode = need_commit && need_decode && !ctx->gc_weighted && decode_commits(ctx->P);
   if (need_commit) {
-    // K4 commit into the stores
-    CommitArgs cm;
+    // K4 commit into the stores (in the decode's launch where it can)
     cm.partials = ctx->partials; cm.P = ctx->P; cm.e_item0 = ph.d_e_item0; cm.e_scale = ph.d_e_scale;
     cm.e_dest = ph.d_e_dest; cm.ndest = ph.ndest; cm.nE = (int)ph.parts.size(); cm.store = ctx->store;
-    nl[PGC_KCOMMIT] = 1;
-    PGC_CK(ctx, launch_commit(cm, st, ctx->pdl));
+    if (!commit_in_decode) {
+      nl[PGC_KCOMMIT] = 1;
+      PGC_CK(ctx, launch_commit(cm, st, ctx->pdl));
+    }
   }
   PGC_CK(ctx, record_event(ctx));
   if (need_decode && ctx->gc_weighted) {
@@ -1312,7 +1315,7 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
   } else if (need_decode) {
     // K5+K6 decode + SGD
     nl[PGC_KDECODE] = 1;
-    PGC_CK(ctx, launch_decode(dc, st, ctx->pdl, ctx->sm_count));
+    PGC_CK(ctx, launch_decode(dc, commit_in_decode ? &cm : nullptr, st, ctx->pdl, ctx->sm_count));
   }
   PGC_CK(ctx, record_event(ctx));
   if (ctx->timing) {

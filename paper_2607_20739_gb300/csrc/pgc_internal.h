@@ -124,7 +124,9 @@ struct CommitArgs {
 };
 cudaError_t launch_commit(const CommitArgs& a, cudaStream_t st, bool pdl = false);
 
-cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t st, bool pdl, int sm_count);
+// cm (only if decode_commits(P)): the step's commit, done by the decode for the same columns
+bool decode_commits(int64_t P);
+cudaError_t launch_decode(const DecodeArgs& a, const CommitArgs* cm, cudaStream_t st, bool pdl, int sm_count);
 
 // ---- GC-CR coding: the naive pipelined construction and GC-CR (§V-A) -------
 constexpr int kGcMaxN = 64;   // workers of the GC-CR modes (one-warp fp64 solves)

@@ -9,7 +9,7 @@
 //                     1/n; §V-B CR: every received coded gradient, times
 //                     1/(n mu) = 1/((n-s)c)).
 //   decode_columns /  ghat = B * sum_o U[o] + sum_{stores r with b_r != B}
-//   decode_chunks     (b_r - B) * sum_o store[r][o], fused with the SGD update
+//   decode_chunk      (b_r - B) * sum_o store[r][o], fused with the SGD update
 //                     beta <- beta - eta * ghat (§III); U[o_t] is refreshed.
 //
 // Decode arithmetic.  Coded gradient of store r: C_r = sum_o store[r][o]
@@ -292,67 +292,121 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
   }
 }
 
-// Decode + SGD over chunks q0, q0 + qstride, ... of kDecX float4 columns, the
-// stores split over kDecY thread rows (for large P, many CTAs).  Must be
-// called by exactly kDecX * kDecY threads, all of which pass every bar().
+// Decode + SGD of kDecX float4 columns (chunk q), their terms split over kDecY
+// thread rows (for large P, many CTAs).  Must be called by exactly
+// kDecX * kDecY threads, all of which pass every bar().  red: [2 kDecY][kDecX].
+// Steady steps: each thread row sums its share of the refreshed slot's stores
+// (the new U[o_t]) and, with their coefficients, of the other slot totals and
+// the deviating stores' slots, all loads of a column in flight over the rows;
+// one exchange.  (One slot after the other, with two barriers each, a step of
+// 12 x 4096 x 3072, K = 100 spent 21 us here, now 16.)
 constexpr int kDecX = 32;
 constexpr int kDecY = 8;
 
 template <class Bar>
-__device__ void decode_chunks(const DecodeArgs& a, const DecodePlan& pl, float4 (*red)[kDecX], int tid, int64_t q0,
-                              int64_t qstride, Bar bar) {
+__device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (*red)[kDecX], int tid, int64_t q,
+                             Bar bar) {
   const int x = tid % kDecX, y = tid / kDecX;
   const int64_t P4 = a.P / 4;
-  const int64_t nq = (P4 + kDecX - 1) / kDecX;
   const int c = a.c;
   const float B = pl.B;
   const int ndev = pl.ndev;
   const float4* store = reinterpret_cast<const float4*>(a.store);
   float4* U = reinterpret_cast<float4*>(a.U);
-  for (int64_t q = q0; q < nq; q += qstride) {
-    const int64_t p = q * kDecX + x;
-    const bool inb = p < P4;
-    float4 V = f4zero();
-    for (int o = 0; o < c; ++o) {
-      if (a.slot < 0 || (o == a.slot && !a.u_ready)) {
-        float4 part = f4zero();
-        if (inb)
-          for (int r = y; r < a.owners; r += kDecY) part = f4add(part, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
-        red[y][x] = part;
-        bar();
-        if (y == 0) {
-          float4 u = red[0][x];
+  const int64_t p = q * kDecX + x;
+  const bool inb = p < P4;
+  if (a.slot >= 0) {
+    float4 un = f4zero(), rest = f4zero();
+    if (inb) {
+      if (!a.u_ready) {
+        const float4* s0 = store + (int64_t)a.slot * P4 + p;
+        for (int r0 = y; r0 < a.owners; r0 += 4 * kDecY) {
+          float4 v[4];
 #pragma unroll
-          for (int j = 1; j < kDecY; ++j) u = f4add(u, red[j][x]);
-          if (inb) U[(int64_t)o * P4 + p] = u;
-          V = f4add(V, u);
+          for (int j = 0; j < 4; ++j)
+            v[j] = r0 + j * kDecY < a.owners ? __ldcg(s0 + (int64_t)(r0 + j * kDecY) * c * P4) : f4zero();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) un = f4add(un, v[j]);
         }
-        bar();
-      } else if (y == 0 && inb) {
-        V = f4add(V, __ldcg(U + (int64_t)o * P4 + p));
+      } else if (y == 0) {
+        un = __ldcg(U + (int64_t)a.slot * P4 + p);
+      }
+      // term t: slot total t (t < c, t != o_t), then slot o of deviating store d
+      const int nt = c + ndev * c;
+      for (int t0 = y; t0 < nt; t0 += 4 * kDecY) {
+        float4 v[4];
+        float f[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int t = t0 + j * kDecY;
+          v[j] = f4zero();
+          f[j] = B;
+          if (t < c) {
+            if (t != a.slot) v[j] = __ldcg(U + (int64_t)t * P4 + p);
+          } else if (t < nt) {
+            const int d = (t - c) / c, o = (t - c) - d * c;
+            f[j] = pl.devc[d];
+            v[j] = __ldcg(store + ((int64_t)pl.dev[d] * c + o) * P4 + p);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) rest = f4fma(f[j], v[j], rest);
       }
     }
-    float4 dv = f4zero();
-    if (inb)
-      for (int qq = y; qq < ndev; qq += kDecY) {
-        const int r = pl.dev[qq];
-        float4 Cr = f4zero();
-        for (int o = 0; o < c; ++o) Cr = f4add(Cr, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
-        dv = f4fma(pl.devc[qq], Cr, dv);
-      }
-    red[y][x] = dv;
+    red[y][x] = un;
+    red[kDecY + y][x] = rest;
     bar();
     if (y == 0 && inb) {
-      float4 D = red[0][x];
 #pragma unroll
-      for (int j = 1; j < kDecY; ++j) D = f4add(D, red[j][x]);
-      const float4 g = f4fma(B, V, D);
+      for (int j = 1; j < kDecY; ++j) {
+        un = f4add(un, red[j][x]);
+        rest = f4add(rest, red[kDecY + j][x]);
+      }
+      if (!a.u_ready) U[(int64_t)a.slot * P4 + p] = un;
+      const float4 g = f4fma(B, un, rest);
       float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       w = f4fma(-a.lr, g, w);
       store_outputs_any(a, p, g, w);
     }
     bar();
+    return;
   }
+  float4 V = f4zero();
+  for (int o = 0; o < c; ++o) {
+    float4 part = f4zero();
+    if (inb)
+      for (int r = y; r < a.owners; r += kDecY) part = f4add(part, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
+    red[y][x] = part;
+    bar();
+    if (y == 0) {
+      float4 u = red[0][x];
+#pragma unroll
+      for (int j = 1; j < kDecY; ++j) u = f4add(u, red[j][x]);
+      if (inb) U[(int64_t)o * P4 + p] = u;
+      V = f4add(V, u);
+    }
+    bar();
+  }
+  float4 dv = f4zero();
+  if (inb)
+    for (int qq = y; qq < ndev; qq += kDecY) {
+      const int r = pl.dev[qq];
+      float4 Cr = f4zero();
+      for (int o = 0; o < c; ++o) Cr = f4add(Cr, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
+      dv = f4fma(pl.devc[qq], Cr, dv);
+    }
+  red[y][x] = dv;
+  bar();
+  if (y == 0 && inb) {
+    float4 D = red[0][x];
+#pragma unroll
+    for (int j = 1; j < kDecY; ++j) D = f4add(D, red[j][x]);
+    const float4 g = f4fma(B, V, D);
+    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
+    w = f4fma(-a.lr, g, w);
+    store_outputs_any(a, p, g, w);
+  }
+  bar();
 }
 
 }  // namespace pgc
