@@ -162,7 +162,7 @@ struct pgc_ctx {
   bool split = false;        // softmax in single precision on the tensor cores
   int sp_nc = 0;             // its clusters of two CTAs
   int sp_Kp = 0, sp_C3 = 0;  // classes padded to 16, columns of R
-  int sp_chunk = 0;          // K blocks per accumulator
+  int sp_h = kSplitTile;     // rows per CTA and logits unit
   uint16_t* R3 = nullptr;    // residual parts [R rows][C3]
   void* tmX = nullptr;       // device tensor maps of X: [n] logits, [n] gradient
   alignas(64) unsigned char tmW3[128];   // W parts [3 Kp][ld]
@@ -331,36 +331,58 @@ void build_dynamic_items(pgc_ctx* ctx, Phase& ph, int per_sm) {
   }
 }
 
-// Units of the single-precision tensor-core softmax kernels.  Logits: 256
-// rows of a partition.  Gradient: 256 features of a run of L rows of a
-// partition; L is the multiple of 64 that minimises the rounds over the
-// clusters times a unit's length (its K blocks plus about six for filling the
-// pipeline and writing out), plus the commit of the partials (a launch, and
-// writing and reading them at about 5 TB/s, in blocks of about 0.3 us) that
-// more than one unit per partition and feature tile costs.
+// Row tile height of the logits units: the rounds over the clusters times a
+// unit's time, 64-column blocks of h rows at 45 GB/s per SM (its share of the
+// copy rate) but at least 0.35 us each (MMAs, waits), plus 2 us for its
+// start and epilogue; the largest of the best heights.  From 33 classes on,
+// where every tile reads more of W than of X, more and lower tiles cost more than
+// idle SMs (12 x 4096 x 3072, K = 33: 246 us per step against 229 with full tiles).
+int split_height(const pgc_ctx* ctx, const std::vector<int64_t>& rows) {
+  const int cl = split_cluster(ctx->sp_Kp);
+  int best_h = kSplitTile;
+  if (cl > 1) return best_h;
+  double best = 0.0;
+  for (int h = kSplitTile; h >= 32; h -= 8) {
+    int64_t units = 0;
+    for (int64_t m : rows) units += (m + cl * h - 1) / (cl * h);
+    const double block = std::max(0.35, h * 64.0 * (double)ctx->esize / 45e3);
+    const double cost = (double)((units + ctx->sp_nc - 1) / ctx->sp_nc) * (block * (double)(ctx->ld / 64) + 2.0);
+    if (h == kSplitTile || cost < 0.999 * best) { best = cost; best_h = h; }
+  }
+  return best_h;
+}
+
+// Units of the single-precision tensor-core softmax kernels.  Logits: sp_h
+// rows per CTA of a partition.  Gradient: 128 features per CTA of a run of L rows
+// of a partition; L is the multiple of 64 that minimises the rounds over the
+// clusters times a unit's time (its blocks, modelled as above, and 3 us),
+// plus what more than one unit per partition and feature tile costs: partials
+// written and read again at about 5 TB/s.
 void build_split_units(pgc_ctx* ctx, Phase& ph) {
   const int nE = (int)ph.parts.size();
-  const int64_t SP = (ctx->ld + kSplitFeatures - 1) / kSplitFeatures, nc = ctx->sp_nc;
+  const int cl = split_cluster(ctx->sp_Kp), width = cl * kSplitTile;
+  const int64_t SP = (ctx->ld + width - 1) / width, nc = ctx->sp_nc;
+  // R rows by partition, the same in every phase: the rows between partitions stay zero
+  std::vector<int32_t> z0(ctx->n);
   int64_t z = 0;
-  std::vector<int32_t> z0(nE);
-  for (int e = 0; e < nE; ++e) {
-    const int64_t m = ph.e_rows[e];
-    z0[e] = (int32_t)z;
-    for (int64_t r = 0; r < m; r += kSplitRows)
-      ph.sl_units.push_back({e, ph.parts[e], (int32_t)ph.e_row0[e], (int32_t)r, (int32_t)m, z0[e], 0, 0});
-    z += (m + 127) / 128 * 128;
+  for (int k = 0; k < ctx->n; ++k) {
+    z0[k] = (int32_t)z;
+    z += (ctx->rows[k] + 127) / 128 * 128;
   }
   ph.zpad_total = z;
+  for (int e = 0; e < nE; ++e)
+    for (int64_t r = 0; r < ph.e_rows[e]; r += cl * ctx->sp_h)
+      ph.sl_units.push_back({e, ph.parts[e], (int32_t)ph.e_row0[e], (int32_t)r, (int32_t)ph.e_rows[e], z0[ph.parts[e]], 0, 0});
+  const double block = std::max(0.35, kSplitTile * 64.0 * (double)ctx->esize / 45e3);
   int64_t best_L = (ph.max_rows + 63) / 64 * 64;
   double best = 0.0;
-  for (int64_t q = 1; q <= 64; ++q) {
+  for (int64_t q = 1; q <= 128; ++q) {
     const int64_t L = ((ph.max_rows + q - 1) / q + 63) / 64 * 64;
-    if (q > 1 && L < 256) break;
+    if (q > 1 && L < 128) break;
     int64_t items = 0;
     for (int e = 0; e < nE; ++e) items += (ph.e_rows[e] + L - 1) / L;
-    const double rounds = (double)((items * SP + nc - 1) / nc);
-    const double commit = items > nE ? 10.0 + (double)items * (double)ctx->P * 8.0 / 5e12 / 0.3e-6 : 0.0;
-    const double cost = rounds * ((double)L / 64.0 + 6.0) + commit;
+    const double commit = items > nE ? 1.0 + (double)items * (double)ctx->P * 8.0 / 5e6 : 0.0;
+    const double cost = (double)((items * SP + nc - 1) / nc) * ((double)L / 64.0 * block + 3.0) + commit;
     if (q == 1 || cost < best) { best = cost; best_L = L; }
   }
   int item = 0;
@@ -369,7 +391,7 @@ void build_split_units(pgc_ctx* ctx, Phase& ph) {
     for (int64_t r = 0; r < ph.e_rows[e]; r += best_L, ++item)
       for (int64_t sp = 0; sp < SP; ++sp)
         ph.sg_units.push_back({e, ph.parts[e], (int32_t)sp, (int32_t)r, (int32_t)std::min(best_L, ph.e_rows[e] - r),
-                               z0[e], item, 0});
+                               z0[ph.parts[e]], item, 0});
     ph.e_item0.push_back(item);
   }
   ph.sg_items = item;
@@ -765,7 +787,9 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
       ctx->split = *split = ctx->sp_nc > 0;
       ctx->sp_Kp = split_kp(K);
       ctx->sp_C3 = split_cols(ctx->sp_Kp);
-      ctx->sp_chunk = kSplitChunk;
+      std::vector<int64_t> steady;   // rows of the partitions a steady step evaluates
+      for (int k = 0; k < n; k += scheme == PGC_FR ? ctx->c : 1) steady.push_back(rows[k]);
+      if (ctx->split) ctx->sp_h = split_height(ctx, steady);
     }
   }
   ctx->P = ctx->K * ctx->ld;
@@ -873,7 +897,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   PGC_ALLOC(ctx->partials, max_partials * sizeof(float));
   int64_t max_zpad = 0;
   for (auto& ph : ctx->phases) max_zpad = std::max(max_zpad, ph.zpad_total);
-  if (loss == PGC_SOFTMAX && !no_split && ctx->total_rows < (int64_t(1) << 31) - kSplitRows) {
+  if (loss == PGC_SOFTMAX && !no_split && ctx->total_rows < (int64_t(1) << 31) - 2 * kSplitTile) {
     // the loss on the tensor cores, if the parts of W fit
     const int nc = split_max_clusters(kSplitLoss, dtype, std::min(K, kSplitMaxClasses));
     ctx->lw_Kp = split_kp(std::min(K, kSplitMaxClasses));
@@ -968,6 +992,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   if (e == cudaSuccess && ctx->wb) e = refresh_wb(ctx);
   if (e == cudaSuccess && ctx->lw && ctx->lw != ctx->wb)
     e = cudaMemsetAsync(ctx->lw, 0, (size_t)3 * ctx->lw_ncb * ctx->lw_Kp * ctx->ld * 2, st);
+  if (e == cudaSuccess && ctx->R3) e = cudaMemsetAsync(ctx->R3, 0, (size_t)max_zpad * ctx->sp_C3 * 2, st);
   if (e == cudaSuccess && ctx->Rb) e = cudaMemsetAsync(ctx->Rb, 0, (size_t)max_zpad * ctx->Ktc * 2, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(e);
@@ -1016,7 +1041,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     alignas(64) unsigned char m[128];
     const bool f32 = dtype == PGC_F32;
     if (!make_tmap_2d(ctx->tmWl, false, ctx->lw, ctx->ld, (uint64_t)3 * ctx->lw_ncb * ctx->lw_Kp, (uint64_t)ctx->ld * 2, 64,
-                      (uint32_t)(3 * ctx->lw_Kp / 2), true) ||
+                      (uint32_t)(3 * ctx->lw_Kp / split_cluster(ctx->lw_Kp)), true) ||
         !make_tmap_2d(m, f32, ctx->X, ctx->ld, ctx->total_rows, (uint64_t)ctx->ld * ctx->esize, f32 ? 32 : 64, 128, true))
       return fail(cudaErrorInvalidValue);
     e = cudaMemcpyAsync(ctx->tmXl, m, 128, cudaMemcpyHostToDevice, st);
@@ -1026,15 +1051,16 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   if (ctx->split) {
     // X through one map per partition: rows past it read as zero
     const bool f32 = dtype == PGC_F32;
+    const uint32_t cl = (uint32_t)split_cluster(ctx->sp_Kp);
     const uint64_t pitch = (uint64_t)ctx->ld * ctx->esize;
     std::vector<uint8_t> maps((size_t)2 * n * 128 + 64);
     uint8_t* m = reinterpret_cast<uint8_t*>(align_up(reinterpret_cast<uintptr_t>(maps.data()), 64));
     bool ok = make_tmap_2d(ctx->tmW3, false, ctx->wb, ctx->ld, 3 * ctx->sp_Kp, (uint64_t)ctx->ld * 2, 64,
-                           (uint32_t)(3 * ctx->sp_Kp / 2), true) &&
-              make_tmap_2d(ctx->tmR3, false, ctx->R3, ctx->sp_C3, max_zpad, (uint64_t)ctx->sp_C3 * 2, 64, 32, true);
+                           (uint32_t)(3 * ctx->sp_Kp / cl), true) &&
+              make_tmap_2d(ctx->tmR3, false, ctx->R3, ctx->sp_C3, max_zpad, (uint64_t)ctx->sp_C3 * 2, 64, 64 / cl, true);
     for (int k = 0; k < n && ok; ++k) {
       const uint8_t* Xk = static_cast<const uint8_t*>(ctx->X) + (size_t)ctx->row0[k] * pitch;
-      ok = make_tmap_2d(m + (size_t)k * 128, f32, Xk, ctx->ld, ctx->rows[k], pitch, f32 ? 32 : 64, 128, true) &&
+      ok = make_tmap_2d(m + (size_t)k * 128, f32, Xk, ctx->ld, ctx->rows[k], pitch, f32 ? 32 : 64, (uint32_t)ctx->sp_h, true) &&
            make_tmap_2d(m + (size_t)(n + k) * 128, f32, Xk, ctx->ld, ctx->rows[k], pitch, f32 ? 128 : 64, 64, !f32);
     }
     if (!ok) return fail(cudaErrorInvalidValue);
@@ -1268,7 +1294,7 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
   } else if (ctx->split) {
     SplitArgs a = {};
     a.K = (int)ctx->K; a.Kp = ctx->sp_Kp; a.C3 = ctx->sp_C3; a.ld = ctx->ld; a.P = ctx->P;
-    a.nkb = (int)(ctx->ld / 64); a.chunk = ctx->sp_chunk;
+    a.nkb = (int)(ctx->ld / 64); a.cl = split_cluster(a.Kp); a.h = ctx->sp_h; a.chunk = split_chunk(a.Kp);
     a.R3 = ctx->R3; a.y = static_cast<const int32_t*>(ctx->y); a.partials = ctx->partials;
     a.e_scale = ph.d_e_scale; a.e_dest = ph.d_e_dest; a.ndest = ph.ndest; a.store = ctx->store;
     a.status = ctx->status;
@@ -1360,9 +1386,10 @@ int pgc_loss(pgc_ctx* ctx, double* loss_out) {
     if (ctx->lw != ctx->wb) PGC_CK(ctx, launch_split_weights(ctx->w, ctx->lw, ctx->K, ctx->ld, ctx->lw_Kp, ctx->stream));
     SplitArgs a = {};
     a.K = (int)ctx->K; a.Kp = ctx->lw_Kp; a.ncb = ctx->lw_ncb; a.ld = ctx->ld; a.nkb = (int)(ctx->ld / 64);
-    a.chunk = kSplitChunk; a.tmX = ctx->tmXl; a.rows = ctx->total_rows;
+    a.cl = split_cluster(a.Kp); a.h = kSplitTile; a.chunk = split_chunk(a.Kp);
+    a.tmX = ctx->tmXl; a.rows = ctx->total_rows;
     a.row_stats = ctx->row_stats; a.row_lab = ctx->row_lab;
-    a.nunits = ctx->lw_ncb * (int)((ctx->total_rows + kSplitRows - 1) / kSplitRows);
+    a.nunits = ctx->lw_ncb * (int)((ctx->total_rows + a.cl * a.h - 1) / (a.cl * a.h));
     a.y = static_cast<const int32_t*>(ctx->y); a.status = ctx->status;
     PGC_CK(ctx, launch_split(kSplitLoss, ctx->dtype, ctx->tmWl, a, ctx->lw_nc, ctx->pdl, ctx->stream));
     PGC_CK(ctx, launch_loss_combine(ctx->row_stats, ctx->row_lab, ctx->total_rows, ctx->lw_ncb, ctx->loss_blocks,

@@ -375,15 +375,15 @@ bool make_tmap_bf16_rows(void* tm_out, const void* base, uint64_t ld, uint64_t r
 // the MMA's N axis (3 Kp columns), fp32 X cut into three parts in the kernel.
 constexpr int64_t kSplitMaxClasses = 128;
 enum { kSplitLogits = 0, kSplitGrad = 1, kSplitLoss = 2 };   // kernels (launch_split's mode)
-constexpr int kSplitChunk = 2;             // 64-wide K blocks per leading accumulator
-constexpr int kSplitRows = 256;            // rows of X per logits unit (two CTAs of 128)
-constexpr int kSplitFeatures = 256;        // features per gradient unit (two CTAs of 128)
+constexpr int kSplitTile = 128;            // rows (logits) or features (gradient) of a CTA at most
 inline int split_kp(int64_t K) { return (int)((K + 15) / 16 * 16); }
+inline int split_cluster(int Kp) { return Kp <= 32 ? 1 : 2; }       // CTAs that share the B tiles
+inline int split_chunk(int Kp) { return Kp <= 32 ? 2 : 4; }         // 64-wide K blocks per leading accumulator
 inline int split_cols(int Kp) { return (3 * Kp + 63) / 64 * 64; }   // columns of R
 struct SplitUnit {
   int32_t e;      // position of the partition in the phase's evaluated list
   int32_t map;    // its tensor map (partition index)
-  int32_t x;      // logits: first global row of the partition (labels); gradient: 256-feature tile
+  int32_t x;      // logits: first global row of the partition (labels); gradient: tile of 128 cl features
   int32_t r0;     // first row of the unit within the partition
   int32_t rows;   // logits: rows of the partition; gradient: rows of the unit (from r0)
   int32_t z0;     // first R row of the partition (a multiple of 128)
@@ -395,6 +395,8 @@ struct SplitArgs {
   int nunits;
   const void* tmX;          // device array of tensor maps, one per partition
   int nkb;                  // logits: ld / 64
+  int cl;                   // CTAs per cluster (split_cluster)
+  int h;                    // logits, loss: rows per CTA and unit, the row box of tmX
   int chunk;                // K blocks of 64 per accumulator before it is added up in fp32
   int K, Kp, C3;            // classes, padded to 16, columns of R (split_cols)
   int64_t ld, P;
@@ -406,7 +408,7 @@ struct SplitArgs {
   int ndest;
   float* store;
   int* status;
-  // loss: nunits = ncb x ceil(rows / 256) units over all rows (one map), class
+  // loss: nunits = ncb x ceil(rows / (cl h)) units over all rows (one map), class
   // block n % ncb of row tile n / ncb; (max, sum of exp) per block and row, label logits
   int64_t rows;
   int ncb;
@@ -415,9 +417,9 @@ struct SplitArgs {
 };
 // Clusters of two CTAs that fit at once (0: cannot launch).
 int split_max_clusters(int mode, int dtype, int64_t K);
-// kSplitLogits: R from X and W; tmB = W parts [3 Kp][ld], box {64, 3 Kp / 2}; tmX: box
-// {128 bytes, 128} per partition, 128-byte swizzle.  kSplitGrad: partials (or stores) from R and X;
-// tmB = R [rows][C3], box {64, 32}; tmX: bf16 box {64, 64}, 128-byte swizzle; fp32 box {128, 64}, no swizzle.
+// kSplitLogits: R from X and W; tmB = W parts [3 Kp][ld], box {64, 3 Kp / cl}; tmX: box
+// {128 bytes, h} per partition, 128-byte swizzle.  kSplitGrad: partials (or stores) from R and X;
+// tmB = R [rows][C3], box {64, 64 / cl}; tmX: bf16 box {64, 64}, 128-byte swizzle; fp32 box {128, 64}, no swizzle.
 // kSplitLoss: tmB = W parts [ncb][3 Kp][ld]; tmX: one map over all rows, box as kSplitLogits.
 cudaError_t launch_split(int mode, int dtype, const void* tmB, const SplitArgs& a, int nclusters, bool pdl,
                          cudaStream_t st);

@@ -19,22 +19,25 @@
 // The tensor core cuts a sum off (it does not round it) at every K step, so a
 // long sum drifts: one leading accumulator over all 4096 rows (3072 features)
 // left the gradient 4.7e-6 off, 9.2e-7 with the CUDA-core sums.  So the
-// leading accumulator is emptied into fp32 registers every `chunk` = 2 stages
-// (128 products; 2.0e-7; 3.2e-7 with 4 stages, 6.0e-7 with 8), alternating
-// with a second one where tensor memory has room.
+// leading accumulator is emptied into fp32 registers every two stages (128
+// products; 2.0e-7), from 33 classes on every four (3.2e-7; 6.0e-7 with eight),
+// alternating with a second one where tensor memory has room.
 //
 // Measured, us per step, before (three CUDA-core kernels) and with this file:
-// 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 286; 8 of 4096 x 784
-// fp32, 10 classes: 915 -> 107.  X is read once per kernel (twice per step);
-// the stages' latency bounds both kernels (2.2-2.9 TB/s of X).
+// 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 228; 8 of 4096 x 784
+// fp32, 10 classes: 915 -> 69.  X is read once per kernel (twice per step).  The
+// instructions of the single-thread roles bound an earlier form (282 and 102,
+// with ring positions divided out and descriptors rebuilt for every MMA).
 //
-// Both kernels are one GEMM skeleton (kGrad selects): a cluster of two CTAs
-// takes units of 256 rows of X (logits; 128 per CTA, the MMA's M) or 256
-// features (gradient; 128 per CTA) and streams its A tiles, 64 columns (rows)
-// a stage, through a ring of TMA stages; the B tiles (W: 3 Kp x 64, K-major; R:
-// 64 rows x 3 Kp, MN-major) are common to the two CTAs, each loads half and
-// multicasts it.  X is read through one tensor map per partition, so that rows
-// past the partition read as zero and never as the next partition's.
+// Both kernels are one GEMM skeleton (kMode selects): a cluster of one or two
+// CTAs takes units of h rows of X per CTA (logits; h <= 128, the MMA's M, chosen so
+// that every SM streams about the same rows) or of 128 features per CTA
+// (gradient) and streams its A tiles, 64 columns (rows) a stage, through a ring of
+// TMA stages, with the B tile (W: 3 Kp x 64, K-major; R: 64 rows x 3 Kp,
+// MN-major).  From 33 classes on, where B outweighs A, two CTAs share it: each
+// loads half and multicasts it.  X is read through one tensor map per
+// partition, so that rows past the partition read as zero and never as the next
+// partition's.
 //   bf16 X: the MMA reads A from the stage (K-major; gradient: MN-major).
 //   fp32 X: eight (four) warps cut a stage's A tile into parts and put them into
 //           tensor memory (one lane per row, or per feature), 32 K elements
@@ -82,10 +85,13 @@ template <typename T, int NCH> constexpr int split_conv() { return sizeof(T) == 
 template <typename T, int NCH> constexpr int split_threads() { return 192 + 32 * split_conv<T, NCH>(); }
 template <typename T> constexpr uint32_t split_a_bytes() { return kSM * kSK * sizeof(T); }
 
-// Tensor memory: nmain accumulators of the leading products (Kp columns),
-// ncorr of the corrections (2 Kp), A buffers from the top.
+// Tensor memory, A buffers from the top.  Up to 32 classes (stack): two
+// accumulators of 3 Kp columns, leading products and corrections side by side, so
+// one MMA multiplies x1 with all parts; more: nmain accumulators of the leading
+// products (Kp columns), ncorr of the corrections (2 Kp).
 struct SplitGeom {
   int stages, nmain, ncorr, nbuf;
+  bool stack;
   uint32_t b_bytes;                            // B tile, a multiple of 1 KB
 };
 // nb: 3 Kp (logits: rows of W) or 3 Kp rounded up to 64 (gradient: columns of R)
@@ -96,6 +102,7 @@ __host__ __device__ inline SplitGeom split_geom(int esize, int Kp, int nb) {
   g.stages = (int)(kSSmemBudget / stage);
   if (g.stages > kSMaxStages) g.stages = kSMaxStages;
   const int room = (int)kSTmem - (esize == 4 ? 2 * (int)kSBufCols : 0);
+  g.stack = Kp <= 32;
   g.nmain = 4 * Kp <= room ? 2 : 1;
   g.ncorr = 6 * Kp <= room ? 2 : 1;
   g.nbuf = esize == 4 ? ((int)kSTmem - (g.nmain + 2 * g.ncorr) * Kp) / (int)kSBufCols : 0;
@@ -185,11 +192,13 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_rank();
+  constexpr bool kStack = NCH == 1;        // split_geom's stack
+  constexpr int CL = kStack ? 1 : 2;       // CTAs of the cluster (split_cluster)
   constexpr uint16_t kBoth = 0x3;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 2);           // both CTAs' MMAs have read the stage
+      mbar_init(&empty[s], CL);          // every CTA's MMAs have read the stage
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
@@ -217,118 +226,156 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
   if (threadIdx.x == 0) grid_dep_launch();
   grid_dep_wait();                       // W (R) is the previous kernel's output
 
-  const int ncl = (int)gridDim.x >> 1, cid = (int)blockIdx.x >> 1;
+  const int ncl = (int)gridDim.x / CL, cid = (int)blockIdx.x / CL;
   // loss: unit = class block e of a row tile, the blocks of a tile side by side
   const int my_units = p.nunits > cid ? (p.nunits - cid + ncl - 1) / ncl : 0;
   auto unit = [&](int i) {
     const int n = cid + i * ncl;
-    if constexpr (kMode == kSplitLoss) return SplitUnit{n % p.ncb, 0, 0, n / p.ncb * kSplitRows, (int)p.rows, 0, 0, 0};
+    if constexpr (kMode == kSplitLoss) return SplitUnit{n % p.ncb, 0, 0, n / p.ncb * CL * p.h, (int)p.rows, 0, 0, 0};
     else return p.units[n];
   };
   auto blocks_of = [&](const SplitUnit& u) { return kGrad ? (u.rows + kSK - 1) / kSK : p.nkb; };
 
   if (warp == 0 && lane == 0) {
     // ---- producer ----------------------------------------------------------
-    int it = 0;
+    // (ring positions and phases are counted, not divided out: the single-thread
+    // roles' instructions are on every stage's critical path)
+    const uint32_t a_bytes = kGrad ? kABytes : (uint32_t)p.h * kSK * (uint32_t)sizeof(T);
+    const int part = 3 * Kp / CL;
+    int it = 0, s = 0;
+    uint32_t ph = 1;                                         // phase of the empty barrier: passes at once in the first round
     bool ok = true;
     for (int i = 0; i < my_units && ok; ++i) {
       const SplitUnit u = unit(i);
       const CUtensorMap* tmA = reinterpret_cast<const CUtensorMap*>(p.tmX) + u.map;
       const int nkb = blocks_of(u);
+      const int r0 = u.r0 + (kGrad ? 0 : rank * p.h), f0 = (CL * u.x + rank) * kSM;
+      const int wrow = (kMode == kSplitLoss ? u.e * 3 * Kp : 0) + rank * part;
       for (int kb = 0; kb < nkb; ++kb, ++it) {
-        const int s = it % S;
-        if (it >= S && !mbar_wait(&empty[s], ((it / S) - 1) & 1, p.status)) { ok = false; break; }
+        if (it >= S && !mbar_wait(&empty[s], ph, p.status)) { ok = false; break; }
         uint8_t* a_dst = sm + (size_t)s * stage_bytes;
         uint8_t* b_dst = a_dst + kABytes;
-        mbar_arrive_expect_tx(&full[s], kABytes + G.b_bytes);
+        mbar_arrive_expect_tx(&full[s], a_bytes + G.b_bytes);
         if constexpr (!kGrad) {
-          const int r = u.r0 + rank * kSM;
-          tma_load_2d(a_dst, tmA, kb * kSK, r, &full[s]);
-          if (kF32) tma_load_2d(a_dst + kABytes / 2, tmA, kb * kSK + 32, r, &full[s]);
-          const int half = 3 * Kp / 2;
-          const int row = (kMode == kSplitLoss ? u.e * 3 * Kp : 0) + rank * half;
-          tma_load_2d_mc(b_dst + (size_t)rank * half * 128, &tmB, kb * kSK, row, &full[s], kBoth);
+          tma_load_2d(a_dst, tmA, kb * kSK, r0, &full[s]);
+          if (kF32) tma_load_2d(a_dst + kABytes / 2, tmA, kb * kSK + 32, r0, &full[s]);
+          if (CL == 1) tma_load_2d(b_dst, &tmB, kb * kSK, wrow, &full[s]);
+          else tma_load_2d_mc(b_dst + (size_t)rank * part * 128, &tmB, kb * kSK, wrow, &full[s], kBoth);
         } else {
-          const int f = (2 * u.x + rank) * kSM, r = u.r0 + kb * kSK;
-          tma_load_2d(a_dst, tmA, f, r, &full[s]);
-          if (!kF32) tma_load_2d(a_dst + kABytes / 2, tmA, f + 64, r, &full[s]);
-          for (int q = 0; q < nb / 64; ++q)
-            tma_load_2d_mc(b_dst + q * 8192 + rank * 4096, &tmB, q * 64, u.z0 + r + rank * 32, &full[s], kBoth);
+          const int r = r0 + kb * kSK;
+          tma_load_2d(a_dst, tmA, f0, r, &full[s]);
+          if (!kF32) tma_load_2d(a_dst + kABytes / 2, tmA, f0 + 64, r, &full[s]);
+          for (int q = 0; q < nb / 64; ++q) {
+            if (CL == 1) tma_load_2d(b_dst + q * 8192, &tmB, q * 64, u.z0 + r, &full[s]);
+            else tma_load_2d_mc(b_dst + q * 8192 + rank * 4096, &tmB, q * 64, u.z0 + r + rank * 32, &full[s], kBoth);
+          }
         }
+        if (++s == S) { s = 0; ph ^= 1u; }
       }
     }
-    for (int s = 0; s < S && s < it; ++s) {   // no copy may outlive the CTA
-      const int last = ((it - 1 - s) / S) * S + s;
-      mbar_wait(&full[s], (last / S) & 1, p.status);
+    // no copy may outlive the CTA
+    for (int q = 0; q < S && q < it; ++q) {
+      const int last = ((it - 1 - q) / S) * S + q;
+      mbar_wait(&full[q], (last / S) & 1, p.status);
     }
   } else if (warp == 1 && lane == 0) {
     // ---- MMA issuer --------------------------------------------------------
-    const uint32_t idesc0 = idesc_bf16_f32(kSM, 0, kGrad && !kF32, kGrad);
+    constexpr uint32_t idesc0 = idesc_bf16_f32(kSM, 0, kGrad && !kF32, kGrad);
     auto idesc = [&](int N) { return idesc0 | ((uint32_t)(N >> 3) << 17); };
-    const uint32_t id1 = idesc(Kp), id2 = idesc(2 * Kp);
+    const uint32_t id1 = idesc(Kp), id2 = idesc(2 * Kp), id3 = idesc(kStack ? 3 * Kp : Kp);
     // x1 times parts 2 and 3: columns Kp .. 3 Kp of B.  MN-major, an operand that
     // starts inside a 64-column block must end there: two MMAs if it does not.
     const int na = kGrad && Kp % 64 != 0 && 2 * Kp > 64 - Kp % 64 ? 64 - Kp % 64 : 2 * Kp, nrest = 2 * Kp - na;
     const uint32_t ida = idesc(na), idr = idesc(nrest);
-    int it = 0, ah = 0, tt = 0;
+    // descriptors of stage 0; a stage further is stage_bytes / 16, a K step (16)
+    // 32 bytes along the swizzled row (K-major) or two 8-row groups (MN-major)
+    auto boff = [&](int n) {                                 // column n of B, in 16-byte units
+      return kGrad ? (uint32_t)(n / 64) * 512u + (uint32_t)(n % 64) / 8u : (uint32_t)n * 8u;
+    };
+    constexpr uint32_t kStepA = kGrad ? 128 : 2, kStepB = kGrad ? 128 : 2;
+    const uint32_t base = smem_u32(sm);
+    const uint64_t da0 = smem_desc_sw128(base, kGrad ? 8192 : 16, 1024);
+    const uint64_t db0 = smem_desc_sw128(base + kABytes, kGrad ? 8192 : 16, 1024);
+    const uint32_t bK = boff(Kp), bR = boff(Kp + na), stage16 = stage_bytes / 16;
+    int s = 0, ab = 0, acc = 0, cor = 0, left = 0;           // left: K blocks until the leading accumulator is handed over
+    uint32_t ph = 0, ph_a = 0, ph_acc = 1, ph_cor = 1;       // phases; those of freed accumulators pass at once in the first round
+    int used = 0;                                            // accumulators taken so far (up to 2)
     bool ok = true;
     for (int i = 0; i < my_units && ok; ++i) {
       const SplitUnit u = unit(i);
       const int nkb = blocks_of(u);
-      for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
-        const int ck = kb % p.chunk;
-        const int acc = G.nmain == 2 ? tt & 1 : 0, cor = G.ncorr == 2 ? i & 1 : 0;
-        if (ck == 0) {                                       // earlier uses of the accumulators are drained
-          const int uses = G.nmain == 2 ? tt / 2 : tt, cuses = G.ncorr == 2 ? i / 2 : i;
-          if (uses > 0 && !mbar_wait(&acc_empty[acc], (uses - 1) & 1, p.status)) { ok = false; break; }
-          if (kb == 0 && cuses > 0 && !mbar_wait(&corr_empty[cor], (cuses - 1) & 1, p.status)) { ok = false; break; }
+      left = 0;
+      uint32_t d = 0;
+      const uint32_t dc = tmem + (uint32_t)((G.nmain + 2 * cor) * Kp);
+      if (!kStack) {
+        if (i >= G.ncorr && !mbar_wait(&corr_empty[cor], ph_cor, p.status)) { ok = false; break; }
+        if (++cor == G.ncorr) { cor = 0; ph_cor ^= 1u; }
+      }
+      for (int kb = 0; kb < nkb && ok; ++kb) {
+        bool fresh = false;
+        if (left == 0) {                                     // the next leading accumulator, drained
+          if (used >= G.nmain && !mbar_wait(&acc_empty[acc], ph_acc, p.status)) { ok = false; break; }
+          if (used < G.nmain) ++used;
+          left = p.chunk;
+          fresh = true;
+          d = tmem + (uint32_t)(acc * (kStack ? 3 * Kp : Kp));
           tc_fence_after();
         }
-        const uint32_t d = tmem + (uint32_t)(acc * Kp), dc = tmem + (uint32_t)((G.nmain + 2 * cor) * Kp);
-        const int s = it % S;
-        if (!mbar_wait(&full[s], (it / S) & 1, p.status)) { ok = false; break; }
-        const uint32_t a_base = smem_u32(sm + (size_t)s * stage_bytes), b_base = a_base + kABytes;
-        // K-major: 32 bytes along the swizzled row per K step; MN-major: two 8-row groups
-        auto bdesc = [&](int kk, int n) {
-          return kGrad ? smem_desc_sw128(b_base + (uint32_t)(n / 64) * 8192u + (uint32_t)(n % 64) * 2u + (uint32_t)kk * 2048u,
-                                         8192, 1024)
-                       : smem_desc_sw128(b_base + (uint32_t)n * 128u + (uint32_t)kk * 32u, 16, 1024);
-        };
+        if (!mbar_wait(&full[s], ph, p.status)) { ok = false; break; }
+        const uint64_t da = da0 + (uint32_t)s * stage16, db = db0 + (uint32_t)s * stage16;
         if constexpr (!kF32) {
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < kSK / 16; ++kk) {
-            const uint64_t da = kGrad ? smem_desc_sw128(a_base + kk * 2048, 8192, 1024)
-                                      : smem_desc_sw128(a_base + kk * 32, 16, 1024);
-            umma_bf16(d, da, bdesc(kk, 0), id1, (ck | kk) != 0 ? 1u : 0u);
-            umma_bf16(dc, da, bdesc(kk, Kp), ida, (kb | kk) != 0 ? 1u : 0u);
-            if (nrest) umma_bf16(dc + (uint32_t)na, da, bdesc(kk, Kp + na), idr, (kb | kk) != 0 ? 1u : 0u);
+            const uint64_t dak = da + kk * kStepA, dbk = db + kk * kStepB;
+            const uint32_t in1 = fresh && kk == 0 ? 0u : 1u;
+            if constexpr (kStack) {
+              umma_bf16(d, dak, dbk, id3, in1);
+            } else {
+              const uint32_t in2 = kb == 0 && kk == 0 ? 0u : 1u;
+              umma_bf16(d, dak, dbk, id1, in1);
+              umma_bf16(dc, dak, dbk + bK, ida, in2);
+              if (nrest) umma_bf16(dc + (uint32_t)na, dak, dbk + bR, idr, in2);
+            }
           }
         } else {
-          for (int h = 0; h < 2; ++h, ++ah) {
-            const int ab = ah % G.nbuf;
-            if (!mbar_wait(&a_full[ab], (ah / G.nbuf) & 1, p.status)) { ok = false; break; }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (!ok) break;
+            if (!mbar_wait(&a_full[ab], ph_a, p.status)) { ok = false; break; }
             tc_fence_after();
             const uint32_t ta = tmem + kSTmem - (uint32_t)(ab + 1) * kSBufCols;
 #pragma unroll
             for (int k2 = 0; k2 < 2; ++k2) {
               const int kk = h * 2 + k2;
               const uint32_t ak = ta + (uint32_t)(k2 * 8);
-              const uint64_t db = bdesc(kk, 0);
-              umma_bf16_ta(d, ak, db, id1, (ck | kk) != 0 ? 1u : 0u);
-              umma_bf16_ta(dc, ak, bdesc(kk, Kp), ida, (kb | kk) != 0 ? 1u : 0u);
-              if (nrest) umma_bf16_ta(dc + (uint32_t)na, ak, bdesc(kk, Kp + na), idr, (kb | kk) != 0 ? 1u : 0u);
-              umma_bf16_ta(dc, ak + 16u, db, id2, 1u);
-              umma_bf16_ta(dc + (uint32_t)Kp, ak + 32u, db, id1, 1u);
+              const uint64_t dbk = db + kk * kStepB;
+              const uint32_t in1 = fresh && kk == 0 ? 0u : 1u;
+              if constexpr (kStack) {
+                umma_bf16_ta(d, ak, dbk, id3, in1);
+                umma_bf16_ta(d + (uint32_t)Kp, ak + 16u, dbk, id2, 1u);
+                umma_bf16_ta(d + (uint32_t)(2 * Kp), ak + 32u, dbk, id1, 1u);
+              } else {
+                const uint32_t in2 = kb == 0 && kk == 0 ? 0u : 1u;
+                umma_bf16_ta(d, ak, dbk, id1, in1);
+                umma_bf16_ta(dc, ak, dbk + bK, ida, in2);
+                if (nrest) umma_bf16_ta(dc + (uint32_t)na, ak, dbk + bR, idr, in2);
+                umma_bf16_ta(dc, ak + 16u, dbk, id2, 1u);
+                umma_bf16_ta(dc + (uint32_t)Kp, ak + 32u, dbk, id1, 1u);
+              }
             }
             umma_commit(&a_empty[ab]);
+            if (++ab == G.nbuf) { ab = 0; ph_a ^= 1u; }
           }
           if (!ok) break;
         }
-        umma_commit_mc(&empty[s], kBoth);
-        if (ck == p.chunk - 1 || kb == nkb - 1) {
+        if (CL == 1) umma_commit(&empty[s]);
+        else umma_commit_mc(&empty[s], kBoth);
+        if (++s == S) { s = 0; ph ^= 1u; }
+        if (--left == 0 || kb == nkb - 1) {
           umma_commit(&acc_full[acc]);
-          ++tt;
+          left = 0;
+          if (++acc == G.nmain) { acc = 0; ph_acc ^= 1u; }
         }
       }
     }
@@ -343,17 +390,18 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
     constexpr int kConv = split_conv<T, NCH>();
     const int q = warp & 3, t = q * 32 + lane;               // row (logits) or feature (gradient)
     const int h0 = kConv == 8 ? (warp - 6) >> 2 : 0;
-    int it = 0;
+    int it = 0, s = 0;
+    uint32_t ph = 0;
     bool ok = true;
     for (int i = 0; i < my_units && ok; ++i) {
       const SplitUnit u = unit(i);
       const int nkb = blocks_of(u);
       for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
-        const int s = it % S;
-        if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (it / S) & 1, p.status))) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.status))) { ok = false; break; }
         const uint8_t* a = sm + (size_t)s * stage_bytes;
+        if (++s == S) { s = 0; ph ^= 1u; }
         for (int h = h0; h < (kConv == 8 ? h0 + 1 : 2); ++h) {
-          const int ah = 2 * it + h, ab = ah % G.nbuf;
+          const uint32_t ah = 2 * (uint32_t)it + (uint32_t)h, use = ah / (uint32_t)G.nbuf, ab = ah - use * (uint32_t)G.nbuf;
           float x[32];
           if constexpr (!kGrad) {
             const uint8_t* row = a + h * (kABytes / 2) + t * 128;
@@ -367,12 +415,12 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
 #pragma unroll
             for (int r = 0; r < 32; ++r) x[r] = col[r * kSM];
           }
-          if (ah >= G.nbuf && !__all_sync(0xffffffffu, mbar_wait(&a_empty[ab], ((ah / G.nbuf) - 1) & 1, p.status))) {
+          if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(&a_empty[ab], (use - 1) & 1u, p.status))) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + kSTmem - (uint32_t)(ab + 1) * kSBufCols;
+          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + kSTmem - (ab + 1) * kSBufCols;
 #pragma unroll
           for (int part = 0; part < 3; ++part) {
             uint32_t w[16];
@@ -406,15 +454,30 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
           break;
         }
         tc_fence_after();
+        if (kStack) {
+          if constexpr (NCH == 1) {
+            float v[32];
 #pragma unroll
-        for (int c = 0; c < NCH * 32; c += 16)
-          if (c < Kp) tmem_add16(lane_base + (uint32_t)(acc * Kp + c), z + c);
+            for (int c = 0; c < 32; ++c) v[c] = 0.f;
+#pragma unroll
+            for (int j = 2; j >= 0; --j)                     // smallest first
+#pragma unroll
+              for (int c = 0; c < 32; c += 16)
+                if (c < Kp) tmem_add16(lane_base + (uint32_t)((acc * 3 + j) * Kp + c), v + c);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) z[c] += v[c];
+          }
+        } else {
+#pragma unroll
+          for (int c = 0; c < NCH * 32; c += 16)
+            if (c < Kp) tmem_add16(lane_base + (uint32_t)(acc * Kp + c), z + c);
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[acc]);
       }
       if (!ok) break;
-      {
+      if (!kStack) {
         // the corrections, 2^-16 and 2^-8 times smaller than the leading sum
         const int cor = G.ncorr == 2 ? i & 1 : 0;
         const uint32_t cb = lane_base + (uint32_t)((G.nmain + 2 * cor) * Kp);
@@ -437,8 +500,8 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
       if constexpr (kMode == kSplitLoss) {
         // this thread's row: max and sum of exp over the class block, the label's
         // logit if it is one of them
-        const int row = u.r0 + rank * kSM + t;
-        if (row < u.rows) {
+        const int row = u.r0 + rank * p.h + t;
+        if (t < p.h && row < u.rows) {
           const int c0 = u.e * Kp, nc = p.K - c0 < Kp ? p.K - c0 : Kp;
           const int lab = p.y[row] - c0;
           float m = -INFINITY, sum = 0.f;
@@ -453,11 +516,11 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
           p.row_stats[(int64_t)u.e * p.rows + row] = make_float2(m, sum);
         }
       } else if constexpr (!kGrad) {
-        // R = softmax(Z) - onehot(y) of this thread's row, zero past the partition
-        const int row = u.r0 + rank * kSM + t;
-        if (u.r0 + rank * kSM < u.rows) {                    // else: no row of this CTA's tile exists
-          const bool valid = row < u.rows;
-          const int lab = valid ? p.y[(int64_t)u.x + row] : -1;
+        // R = softmax(Z) - onehot(y) of this thread's row (rows of R past the
+        // partition, which the gradient's last K block reads, stay zero)
+        const int row = u.r0 + rank * p.h + t;
+        if (t < p.h && row < u.rows) {
+          const int lab = p.y[(int64_t)u.x + row];
           float m = -INFINITY;
 #pragma unroll
           for (int c = 0; c < NCH * 32; ++c)
@@ -479,7 +542,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
               float v[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j)
-                v[j] = valid && c + j < p.K ? (c + j == lab ? -rest : z[c + j]) * inv : 0.f;
+                v[j] = c + j < p.K ? (c + j == lab ? -rest : z[c + j]) * inv : 0.f;
               uint4 p1, p2, p3;
               split8(v, p1, p2, p3);
               *reinterpret_cast<uint4*>(out + c) = p1;
@@ -489,7 +552,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
           }
         }
       } else {
-        const int f = (2 * u.x + rank) * kSM + t;
+        const int f = (CL * u.x + rank) * kSM + t;
         if (f < p.ld) {
           if (u.item >= 0) {
             float* out = p.partials + (int64_t)u.item * p.P + f;
@@ -552,14 +615,14 @@ size_t split_smem(int mode, int dtype, int Kp) {
   return 1024 + (size_t)g.stages * ((size_t)kSM * kSK * es + g.b_bytes);
 }
 
-void split_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int mode, int dtype, int Kp, int clusters) {
+void split_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int mode, int dtype, int Kp, int cl, int clusters) {
   cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * clusters));
+  cfg.gridDim = dim3((unsigned)(cl * clusters));
   cfg.blockDim = dim3((unsigned)(dtype == PGC_BF16 ? split_threads<uint16_t, 1>()
                                                    : Kp <= 64 ? split_threads<float, 2>() : split_threads<float, 4>()));
   cfg.dynamicSmemBytes = split_smem(mode, dtype, Kp);
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = (unsigned)cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -578,7 +641,7 @@ int split_max_clusters(int mode, int dtype, int64_t K) {
     return 0;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  split_config(cfg, attr, mode, dtype, Kp, 1);
+  split_config(cfg, attr, mode, dtype, Kp, split_cluster(Kp), 1);
   int nc = 0;
   return cudaOccupancyMaxActiveClusters(&nc, k, &cfg) == cudaSuccess ? nc : 0;
 }
@@ -593,7 +656,7 @@ cudaError_t launch_split(int mode, int dtype, const void* tmB, const SplitArgs& 
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  split_config(cfg, attr, mode, dtype, a.Kp, nclusters < a.nunits ? nclusters : a.nunits);
+  split_config(cfg, attr, mode, dtype, a.Kp, a.cl, nclusters < a.nunits ? nclusters : a.nunits);
   cfg.stream = st;
   cfg.numAttrs = pdl ? 2 : 1;
   CUtensorMap b;
