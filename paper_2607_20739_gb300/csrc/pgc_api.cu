@@ -748,9 +748,26 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
       ctx->tcf_nc = tc_softmax_max_clusters((int)(ctx->Ktc / 256));
       ctx->tcf = ctx->tcf_nc > 0;
     }
+    // Few classes in bf16: the whole-row kernel reads X once but spends about 0.85 ns
+    // of the grid's time per row on its 16-row tiles, however short the rows; the
+    // split kernels read X twice at 5.3 TB/s.  Fitted to 8 partitions of
+    // 1 MB to 256 MB in all, d = 64 to 3072 (us per step, whole rows / split, K = 10):
+    //   256 MB  d = 64: 1834 / 264   256: 479 / 117   500: 256 / 116   827: 164 / 110
+    //           1024: 137 / 108   1536: 100 / 109   2048: 83 / 113   3072: 70 / 118
+    //   16 MB   d = 64: 120 / 31   256: 38 / 20   500: 27 / 19   827: 23 / 22   1024: 20 / 23
+    //   4 MB    d = 64: 39 / 17   256: 19 / 15   500: 16 / 17   1024: 15 / 19
+    //   1 MB    d = 64: 20 / 16   256: 14 / 16
+    bool few_split = false;
+    if (!ctx->tc && dtype == PGC_BF16 && K <= 16 && allow_split && !no_split && !std::getenv("PGC_NO_ROWS") &&
+        !std::getenv("PGC_NO_ROWS_TAIL")) {
+      const double R = scheme == PGC_FR && mode != PGC_MODE_GC ? (double)ctx->total_rows / ctx->c : (double)ctx->total_rows;
+      const double t_rows = 12.0 + R * std::max(0.85e-3, 0.44e-6 * (double)d);
+      const double t_split = 13.0 + 0.006 * (double)d + R * ((double)d * 2.0 * 0.38e-6 + 0.09e-3);
+      few_split = t_split < 0.95 * t_rows;
+    }
     const char* env2 = std::getenv("PGC_NO_SMALLK");
     const char* env4 = std::getenv("PGC_NO_ROWS");
-    if (!ctx->tc && dtype == PGC_BF16 && !(env2 && env2[0] == '1') && !(env4 && env4[0] == '1') && K <= 16) {
+    if (!ctx->tc && !few_split && dtype == PGC_BF16 && !(env2 && env2[0] == '1') && !(env4 && env4[0] == '1') && K <= 16) {
       // few classes, rows short enough to hold 16 whole rows per CTA pair
       // and slot: one CTA per SM, a cluster of two per tile (PGC_NO_ROWS=1
       // keeps the 8-CTA cluster kernel)
@@ -775,7 +792,8 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
         }
       }
     }
-    if (!ctx->tc && !ctx->smallk && dtype == PGC_BF16 && !(env2 && env2[0] == '1') && smallk_fits(K, ctx->ld)) {
+    if (!ctx->tc && !few_split && !ctx->smallk && dtype == PGC_BF16 && !(env2 && env2[0] == '1') &&
+        smallk_fits(K, ctx->ld)) {
       ctx->sk_nper = (int)((ctx->ld / 64 + 7) / 8);
       ctx->sk_nc = smallk_max_clusters(ctx->sk_nper);
       ctx->smallk = ctx->sk_nc > 0;

@@ -121,3 +121,20 @@ def test_cuda_core_softmax_matches_oracle(libpgc, cuda, monkeypatch, dtype):
     for a, b in zip(recs, run_oracle(w, Xs, ys, masks)):
         assert rel_err(a["grad"], b["grad"]) < TOL
     g.close()
+
+
+@pytest.mark.parametrize("d,m,path", [(64, 2000, "softmax_cc"), (64, 40, "softmax_rows"), (300, 4000, "softmax_cc"),
+                                      (300, 100, "softmax_rows"), (1100, 300, "softmax_rows")])
+@pytest.mark.parametrize("mode", ["pgc", "naive_cr"])
+def test_few_classes_take_the_faster_path(libpgc, cuda, d, m, path, mode):
+    """bf16 with up to 16 classes: whole rows, or split operands where rows are
+    short and many; both against the oracle (whole rows round W and R to bf16)."""
+    w = W.WORKLOADS["fr_n32_softmax_k10"].replace(scheme="CR", n=6, s=2, m=m, d=d)
+    if mode == "pgc":
+        Xs, ys, masks = generate(w, 4)
+        g, recs = run_gpu(libpgc, w, Xs, ys, masks)
+        compare_runs(w, recs, run_oracle(w, Xs, ys, masks))
+    else:
+        g = libpgc.PGC(w.scheme, w.n, w.s, w.loss, w.dtype, w.d, K=w.K, rows=w.rows(), lr=w.lr, mode=mode)
+    assert g.gradient_path == path
+    g.close()
