@@ -24,8 +24,8 @@
 // alternating with a second one where tensor memory has room.
 //
 // Measured, us per step, before (three CUDA-core kernels) and with this file:
-// 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 228; 8 of 4096 x 784
-// fp32, 10 classes: 915 -> 69.  X is read once per kernel (twice per step).  The
+// 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 227; 8 of 4096 x 784
+// fp32, 10 classes: 915 -> 64.  X is read once per kernel (twice per step).  The
 // instructions of the single-thread roles bound an earlier form (282 and 102,
 // with ring positions divided out and descriptors rebuilt for every MMA).
 //
@@ -234,9 +234,25 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
     if constexpr (kMode == kSplitLoss) return SplitUnit{n % p.ncb, 0, 0, n / p.ncb * CL * p.h, (int)p.rows, 0, 0, 0};
     else return p.units[n];
   };
+  // The producer and the MMA issuer run as whole, converged warps (elect_one): 8 to
+  // 11 % of a step with fp32 features (8 x 4096 x 784, K = 10: 67.2 us against 61.8;
+  // 8 x 2000 x 2000, K = 20: 126 against 112), 2 to 3 % in bf16 up to 64 classes.
+  // Not so for more classes in bf16, where one thread each is faster (12 x 4096
+  // x 3072, K = 100: 226 against 233).
+  constexpr bool kWhole = kF32 || NCH <= 2;
+  auto one = [] { return kWhole ? elect_one() : true; };
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    return kWhole ? mbar_wait_warp(bar, parity, p.status) : mbar_wait(bar, parity, p.status);
+  };
+  auto join = [] { if (kWhole) __syncwarp(); };
+  auto uniform = [](const SplitUnit& u) {    // known to be warp-uniform to the compiler
+    if (!kWhole) return u;
+    auto sh = [](int v) { return __shfl_sync(0xffffffffu, v, 0); };
+    return SplitUnit{sh(u.e), sh(u.map), sh(u.x), sh(u.r0), sh(u.rows), sh(u.z0), sh(u.item), 0};
+  };
   auto blocks_of = [&](const SplitUnit& u) { return kGrad ? (u.rows + kSK - 1) / kSK : p.nkb; };
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && (kWhole || lane == 0)) {
     // ---- producer ----------------------------------------------------------
     // (ring positions and phases are counted, not divided out: the single-thread
     // roles' instructions are on every stage's critical path)
@@ -246,39 +262,42 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
     uint32_t ph = 1;                                         // phase of the empty barrier: passes at once in the first round
     bool ok = true;
     for (int i = 0; i < my_units && ok; ++i) {
-      const SplitUnit u = unit(i);
+      const SplitUnit u = uniform(unit(i));
       const CUtensorMap* tmA = reinterpret_cast<const CUtensorMap*>(p.tmX) + u.map;
       const int nkb = blocks_of(u);
       const int r0 = u.r0 + (kGrad ? 0 : rank * p.h), f0 = (CL * u.x + rank) * kSM;
       const int wrow = (kMode == kSplitLoss ? u.e * 3 * Kp : 0) + rank * part;
       for (int kb = 0; kb < nkb; ++kb, ++it) {
-        if (it >= S && !mbar_wait(&empty[s], ph, p.status)) { ok = false; break; }
+        if (it >= S && !wait(&empty[s], ph)) { ok = false; break; }
         uint8_t* a_dst = sm + (size_t)s * stage_bytes;
         uint8_t* b_dst = a_dst + kABytes;
-        mbar_arrive_expect_tx(&full[s], a_bytes + G.b_bytes);
-        if constexpr (!kGrad) {
-          tma_load_2d(a_dst, tmA, kb * kSK, r0, &full[s]);
-          if (kF32) tma_load_2d(a_dst + kABytes / 2, tmA, kb * kSK + 32, r0, &full[s]);
-          if (CL == 1) tma_load_2d(b_dst, &tmB, kb * kSK, wrow, &full[s]);
-          else tma_load_2d_mc(b_dst + (size_t)rank * part * 128, &tmB, kb * kSK, wrow, &full[s], kBoth);
-        } else {
-          const int r = r0 + kb * kSK;
-          tma_load_2d(a_dst, tmA, f0, r, &full[s]);
-          if (!kF32) tma_load_2d(a_dst + kABytes / 2, tmA, f0 + 64, r, &full[s]);
-          for (int q = 0; q < nb / 64; ++q) {
-            if (CL == 1) tma_load_2d(b_dst + q * 8192, &tmB, q * 64, u.z0 + r, &full[s]);
-            else tma_load_2d_mc(b_dst + q * 8192 + rank * 4096, &tmB, q * 64, u.z0 + r + rank * 32, &full[s], kBoth);
+        if (one()) {
+          mbar_arrive_expect_tx(&full[s], a_bytes + G.b_bytes);
+          if constexpr (!kGrad) {
+            tma_load_2d(a_dst, tmA, kb * kSK, r0, &full[s]);
+            if (kF32) tma_load_2d(a_dst + kABytes / 2, tmA, kb * kSK + 32, r0, &full[s]);
+            if (CL == 1) tma_load_2d(b_dst, &tmB, kb * kSK, wrow, &full[s]);
+            else tma_load_2d_mc(b_dst + (size_t)rank * part * 128, &tmB, kb * kSK, wrow, &full[s], kBoth);
+          } else {
+            const int r = r0 + kb * kSK;
+            tma_load_2d(a_dst, tmA, f0, r, &full[s]);
+            if (!kF32) tma_load_2d(a_dst + kABytes / 2, tmA, f0 + 64, r, &full[s]);
+            for (int q = 0; q < nb / 64; ++q) {
+              if (CL == 1) tma_load_2d(b_dst + q * 8192, &tmB, q * 64, u.z0 + r, &full[s]);
+              else tma_load_2d_mc(b_dst + q * 8192 + rank * 4096, &tmB, q * 64, u.z0 + r + rank * 32, &full[s], kBoth);
+            }
           }
         }
+        join();
         if (++s == S) { s = 0; ph ^= 1u; }
       }
     }
     // no copy may outlive the CTA
     for (int q = 0; q < S && q < it; ++q) {
       const int last = ((it - 1 - q) / S) * S + q;
-      mbar_wait(&full[q], (last / S) & 1, p.status);
+      wait(&full[q], (last / S) & 1);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && (kWhole || lane == 0)) {
     // ---- MMA issuer --------------------------------------------------------
     constexpr uint32_t idesc0 = idesc_bf16_f32(kSM, 0, kGrad && !kF32, kGrad);
     auto idesc = [&](int N) { return idesc0 | ((uint32_t)(N >> 3) << 17); };
@@ -300,80 +319,92 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
     int s = 0, ab = 0, acc = 0, cor = 0, left = 0;           // left: K blocks until the leading accumulator is handed over
     uint32_t ph = 0, ph_a = 0, ph_acc = 1, ph_cor = 1;       // phases; those of freed accumulators pass at once in the first round
     int used = 0;                                            // accumulators taken so far (up to 2)
+    auto hand_over = [&](int stage, int a, bool done) {      // the stage is read, the accumulator complete
+      if (CL == 1) umma_commit(&empty[stage]);
+      else umma_commit_mc(&empty[stage], kBoth);
+      if (done) umma_commit(&acc_full[a]);
+    };
     bool ok = true;
     for (int i = 0; i < my_units && ok; ++i) {
-      const SplitUnit u = unit(i);
+      const SplitUnit u = uniform(unit(i));
       const int nkb = blocks_of(u);
       left = 0;
       uint32_t d = 0;
       const uint32_t dc = tmem + (uint32_t)((G.nmain + 2 * cor) * Kp);
       if (!kStack) {
-        if (i >= G.ncorr && !mbar_wait(&corr_empty[cor], ph_cor, p.status)) { ok = false; break; }
+        if (i >= G.ncorr && !wait(&corr_empty[cor], ph_cor)) { ok = false; break; }
         if (++cor == G.ncorr) { cor = 0; ph_cor ^= 1u; }
       }
       for (int kb = 0; kb < nkb && ok; ++kb) {
         bool fresh = false;
         if (left == 0) {                                     // the next leading accumulator, drained
-          if (used >= G.nmain && !mbar_wait(&acc_empty[acc], ph_acc, p.status)) { ok = false; break; }
+          if (used >= G.nmain && !wait(&acc_empty[acc], ph_acc)) { ok = false; break; }
           if (used < G.nmain) ++used;
           left = p.chunk;
           fresh = true;
           d = tmem + (uint32_t)(acc * (kStack ? 3 * Kp : Kp));
           tc_fence_after();
         }
-        if (!mbar_wait(&full[s], ph, p.status)) { ok = false; break; }
+        if (!wait(&full[s], ph)) { ok = false; break; }
         const uint64_t da = da0 + (uint32_t)s * stage16, db = db0 + (uint32_t)s * stage16;
+        const bool done = left == 1 || kb == nkb - 1;        // the accumulator is handed over after this block
         if constexpr (!kF32) {
           tc_fence_after();
+          if (one()) {
 #pragma unroll
-          for (int kk = 0; kk < kSK / 16; ++kk) {
-            const uint64_t dak = da + kk * kStepA, dbk = db + kk * kStepB;
-            const uint32_t in1 = fresh && kk == 0 ? 0u : 1u;
-            if constexpr (kStack) {
-              umma_bf16(d, dak, dbk, id3, in1);
-            } else {
-              const uint32_t in2 = kb == 0 && kk == 0 ? 0u : 1u;
-              umma_bf16(d, dak, dbk, id1, in1);
-              umma_bf16(dc, dak, dbk + bK, ida, in2);
-              if (nrest) umma_bf16(dc + (uint32_t)na, dak, dbk + bR, idr, in2);
+            for (int kk = 0; kk < kSK / 16; ++kk) {
+              const uint64_t dak = da + kk * kStepA, dbk = db + kk * kStepB;
+              const uint32_t in1 = fresh && kk == 0 ? 0u : 1u;
+              if constexpr (kStack) {
+                umma_bf16(d, dak, dbk, id3, in1);
+              } else {
+                const uint32_t in2 = kb == 0 && kk == 0 ? 0u : 1u;
+                umma_bf16(d, dak, dbk, id1, in1);
+                umma_bf16(dc, dak, dbk + bK, ida, in2);
+                if (nrest) umma_bf16(dc + (uint32_t)na, dak, dbk + bR, idr, in2);
+              }
             }
+            hand_over(s, acc, done);
           }
         } else {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (!ok) break;
-            if (!mbar_wait(&a_full[ab], ph_a, p.status)) { ok = false; break; }
+            if (!wait(&a_full[ab], ph_a)) { ok = false; break; }
             tc_fence_after();
             const uint32_t ta = tmem + kSTmem - (uint32_t)(ab + 1) * kSBufCols;
+            if (one()) {
 #pragma unroll
-            for (int k2 = 0; k2 < 2; ++k2) {
-              const int kk = h * 2 + k2;
-              const uint32_t ak = ta + (uint32_t)(k2 * 8);
-              const uint64_t dbk = db + kk * kStepB;
-              const uint32_t in1 = fresh && kk == 0 ? 0u : 1u;
-              if constexpr (kStack) {
-                umma_bf16_ta(d, ak, dbk, id3, in1);
-                umma_bf16_ta(d + (uint32_t)Kp, ak + 16u, dbk, id2, 1u);
-                umma_bf16_ta(d + (uint32_t)(2 * Kp), ak + 32u, dbk, id1, 1u);
-              } else {
-                const uint32_t in2 = kb == 0 && kk == 0 ? 0u : 1u;
-                umma_bf16_ta(d, ak, dbk, id1, in1);
-                umma_bf16_ta(dc, ak, dbk + bK, ida, in2);
-                if (nrest) umma_bf16_ta(dc + (uint32_t)na, ak, dbk + bR, idr, in2);
-                umma_bf16_ta(dc, ak + 16u, dbk, id2, 1u);
-                umma_bf16_ta(dc + (uint32_t)Kp, ak + 32u, dbk, id1, 1u);
+              for (int k2 = 0; k2 < 2; ++k2) {
+                const int kk = h * 2 + k2;
+                const uint32_t ak = ta + (uint32_t)(k2 * 8);
+                const uint64_t dbk = db + kk * kStepB;
+                const uint32_t in1 = fresh && kk == 0 ? 0u : 1u;
+                if constexpr (kStack) {
+                  umma_bf16_ta(d, ak, dbk, id3, in1);
+                  umma_bf16_ta(d + (uint32_t)Kp, ak + 16u, dbk, id2, 1u);
+                  umma_bf16_ta(d + (uint32_t)(2 * Kp), ak + 32u, dbk, id1, 1u);
+                } else {
+                  const uint32_t in2 = kb == 0 && kk == 0 ? 0u : 1u;
+                  umma_bf16_ta(d, ak, dbk, id1, in1);
+                  umma_bf16_ta(dc, ak, dbk + bK, ida, in2);
+                  if (nrest) umma_bf16_ta(dc + (uint32_t)na, ak, dbk + bR, idr, in2);
+                  umma_bf16_ta(dc, ak + 16u, dbk, id2, 1u);
+                  umma_bf16_ta(dc + (uint32_t)Kp, ak + 32u, dbk, id1, 1u);
+                }
               }
+              umma_commit(&a_empty[ab]);
             }
-            umma_commit(&a_empty[ab]);
+            join();
             if (++ab == G.nbuf) { ab = 0; ph_a ^= 1u; }
           }
           if (!ok) break;
+          if (one()) hand_over(s, acc, done);
         }
-        if (CL == 1) umma_commit(&empty[s]);
-        else umma_commit_mc(&empty[s], kBoth);
+        join();
         if (++s == S) { s = 0; ph ^= 1u; }
-        if (--left == 0 || kb == nkb - 1) {
-          umma_commit(&acc_full[acc]);
+        --left;
+        if (done) {
           left = 0;
           if (++acc == G.nmain) { acc = 0; ph_acc ^= 1u; }
         }
@@ -381,8 +412,9 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
     }
     // every MMA has completed before TMEM is released (and, on a failure,
     // before the CTA's shared memory goes away)
-    umma_commit(&drained);
-    mbar_wait(&drained, 0, p.status);
+    if (one()) umma_commit(&drained);
+    join();
+    wait(&drained, 0);
   } else if (kF32 && warp >= 6) {
     // ---- fp32 features: cut a stage's A tile into parts in tensor memory -----
     // Eight warps: each half of a stage (32 K elements, one A buffer) has its

@@ -149,6 +149,21 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cl) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cl) : "memory");
 }
 
+// One lane of a converged warp.  The roles that issue TMA copies and MMAs run as
+// whole warps whose control flow and addresses are warp-uniform, and only the
+// instructions themselves sit behind this election: as `lane == 0` branches the
+// compiler kept every descriptor in per-thread registers and moved it to the
+// uniform ones before each instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// mbar_wait by a whole warp: the same answer for all lanes
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status)) != 0;
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
