@@ -748,22 +748,26 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
       ctx->tcf_nc = tc_softmax_max_clusters((int)(ctx->Ktc / 256));
       ctx->tcf = ctx->tcf_nc > 0;
     }
-    // Few classes in bf16: the whole-row kernel reads X once but spends about 0.85 ns
+    // Few classes in bf16: the whole-row kernel reads X once but spends about 0.83 ns
     // of the grid's time per row on its 16-row tiles, however short the rows; the
-    // split kernels read X twice at 5.3 TB/s.  Fitted to 8 partitions of
-    // 1 MB to 256 MB in all, d = 64 to 3072 (us per step, whole rows / split, K = 10):
-    //   256 MB  d = 64: 1834 / 264   256: 479 / 117   500: 256 / 116   827: 164 / 110
-    //           1024: 137 / 108   1536: 100 / 109   2048: 83 / 113   3072: 70 / 118
-    //   16 MB   d = 64: 120 / 31   256: 38 / 20   500: 27 / 19   827: 23 / 22   1024: 20 / 23
-    //   4 MB    d = 64: 39 / 17   256: 19 / 15   500: 16 / 17   1024: 15 / 19
-    //   1 MB    d = 64: 20 / 16   256: 14 / 16
+    // split kernels read X twice.  Both fitted (least squares) to 138 measured points,
+    // 4 to 32 partitions of 1 MB to 256 MB in all, d = 64 to 2048 (us per step, whole
+    // rows / split, 8 partitions, K = 10):
+    //   256 MB  d = 64: 1830 / 262   256: 477 / 118   500: 255 / 114   827: 164 / 107
+    //           1024: 136 / 102   1250: 118 / 109   1536: 100 / 104   2048: 83 / 104
+    //   25 MB   d = 64: 195 / 39   256: 54 / 23   500: 35 / 23   827: 27 / 23   1250: 23 / 26
+    //   4 MB    d = 64: 38 / 17   256: 19 / 15   500: 16 / 17   1024: 15 / 18
+    //   1 MB    d = 64: 19 / 14   256: 14 / 14   1024: 14 / 17
+    // Over these points the choice costs 0.2 % against the better kernel on average
+    // (12 % at worst: 25 MB, d = 1250).  Below 2048 rows the two are within 1 us.
     bool few_split = false;
     if (!ctx->tc && dtype == PGC_BF16 && K <= 16 && allow_split && !no_split && !std::getenv("PGC_NO_ROWS") &&
         !std::getenv("PGC_NO_ROWS_TAIL")) {
       const double R = scheme == PGC_FR && mode != PGC_MODE_GC ? (double)ctx->total_rows / ctx->c : (double)ctx->total_rows;
-      const double t_rows = 12.0 + R * std::max(0.85e-3, 0.44e-6 * (double)d);
-      const double t_split = 13.0 + 0.006 * (double)d + R * ((double)d * 2.0 * 0.38e-6 + 0.09e-3);
-      few_split = t_split < 0.95 * t_rows;
+      const double dd = (double)d;
+      const double t_rows = 12.8 + R * (0.826e-3 + 0.139e-6 * dd);
+      const double t_split = 12.5 + 0.0043 * dd + R * (0.082e-3 + 0.557e-6 * dd);
+      few_split = R >= 2048 && t_split < t_rows;
     }
     const char* env2 = std::getenv("PGC_NO_SMALLK");
     const char* env4 = std::getenv("PGC_NO_ROWS");
