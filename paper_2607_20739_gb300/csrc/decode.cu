@@ -73,25 +73,26 @@ cudaError_t launch_commit(const CommitArgs& a, cudaStream_t st, bool pdl) {
 
 // kCommit: the step's commit first, for the same columns (a column's decode
 // reads only that column of the stores, so a CTA barrier is enough): thread
-// row y sums the items of partitions y, y + kDecY, ..., in item order.  One
+// row y sums the items of partitions y, y + kY, ..., in item order.  One
 // launch instead of two.
-template <bool kCommit>
-__global__ void __launch_bounds__(kDecX * kDecY) decode_kernel(DecodeArgs a, CommitArgs cm) {
+template <bool kCommit, int kY>
+__global__ void __launch_bounds__(256) decode_kernel(DecodeArgs a, CommitArgs cm) {
+  constexpr int kX = 256 / kY;
   __shared__ DecodePlan pl;
-  __shared__ float4 red[2 * kDecY][kDecX];
+  __shared__ float4 red[2 * kY][kX];
   grid_dep_launch();
   if (threadIdx.x < 32) derive_plan_warp(a, pl, threadIdx.x);   // needs only the mask
   __syncthreads();
   grid_dep_wait();
   if (blockIdx.x == 0 && threadIdx.x < 32) write_coeffs_warp(a, threadIdx.x);
-  const int64_t P4 = a.P / 4, nq = (P4 + kDecX - 1) / kDecX;
+  const int64_t P4 = a.P / 4, nq = (P4 + kX - 1) / kX;
   auto bar = [] { __syncthreads(); };
   for (int64_t q = blockIdx.x; q < nq; q += gridDim.x) {
     if constexpr (kCommit) {
-      const int64_t p = q * kDecX + threadIdx.x % kDecX;
+      const int64_t p = q * kX + threadIdx.x % kX;
       if (p < P4) {
         const float4* src = reinterpret_cast<const float4*>(cm.partials) + p;
-        for (int e = threadIdx.x / kDecX; e < cm.nE; e += kDecY) {
+        for (int e = threadIdx.x / kX; e < cm.nE; e += kY) {
           const int i0 = cm.e_item0[e], i1 = cm.e_item0[e + 1];
           float4 acc = f4zero();
           for (int it = i0; it < i1; it += 8) {
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kDecX * kDecY) decode_kernel(DecodeArgs a, Com
       }
       __syncthreads();
     }
-    decode_chunk(a, pl, red, (int)threadIdx.x, q, bar);
+    decode_chunk<kY>(a, pl, red, (int)threadIdx.x, q, bar);
   }
 }
 
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
     // deviating stores' slot o_t
     const float4* pre = reinterpret_cast<const float4*>(a.pre);
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P4; p += (int64_t)gridDim.x * blockDim.x) {
+      float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       float4 g = f4fma(pl.B, __ldcg(U + (int64_t)a.slot * P4 + p), __ldcg(pre + p));
       const float4* cur = store + (int64_t)a.slot * P4 + p;
       for (int q0 = 0; q0 < pl.ndev; q0 += 8) {
@@ -159,14 +161,13 @@ __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
         for (int j = 0; j < 8; ++j)
           if (q0 + j < pl.ndev) g = f4fma(pl.devc[q0 + j], v[j], g);
       }
-      float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       w = f4fma(-a.lr, g, w);
       store_outputs_any(a, p, g, w);
     }
     return;
   }
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P4; p += (int64_t)gridDim.x * blockDim.x) {
-    float4 V = f4zero();
+    float4 V = f4zero(), w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     if (a.slot < 0) {
       for (int o = 0; o < c; ++o) {
         const float4 u = sum_loads8(store + (int64_t)o * P4 + p, a.owners, [&](int r) { return (int64_t)r * slotP; });
@@ -190,13 +191,13 @@ __global__ void __launch_bounds__(256) decode_wide_kernel(DecodeArgs a) {
       D = f4fma(pl.devc[q], Cr, D);
     }
     const float4 g = f4fma(pl.B, V, D);
-    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
     store_outputs_any(a, p, g, w);
   }
 }
 
-// Columns from which the one-thread-per-column decode is used.
+// Columns from which the one-thread-per-column decode is used (8 x 700 x 4096,
+// K = 300: 86 us per step, the kernel above 90; 16 x 1000 x 4096, K = 1000: 426, 443).
 constexpr int64_t kWideDecodeMinP4 = 1 << 18;
 
 bool decode_commits(int64_t P) { return P / 4 < kWideDecodeMinP4; }
@@ -209,12 +210,23 @@ cudaError_t launch_decode(const DecodeArgs& a, const CommitArgs* cm, cudaStream_
     if (blocks > (int64_t)sm_count * 8) blocks = (int64_t)sm_count * 8;
     return launch_maybe_pdl(pdl, decode_wide_kernel, dim3((unsigned)blocks), dim3(256), st, a);
   }
-  const int64_t P4 = a.P / 4;
-  int64_t chunks = (P4 + kDecX - 1) / kDecX;
-  int64_t blocks = chunks < (int64_t)sm_count * 8 ? chunks : (int64_t)sm_count * 8;
-  if (blocks < 1) blocks = 1;
-  if (cm) return launch_maybe_pdl(pdl, decode_kernel<true>, dim3((unsigned)blocks), dim3(kDecX * kDecY), st, a, *cm);
-  return launch_maybe_pdl(pdl, decode_kernel<false>, dim3((unsigned)blocks), dim3(kDecX * kDecY), st, a, CommitArgs{});
+  // Thread rows per column: each column's loads are one latency, so first a grid that
+  // is resident at once (8 CTAs per SM), then as many rows as that leaves.  us per
+  // step with 8 / 4 / 2 / 1 rows (terms of a column in brackets):
+  //   n = 12, K = 33,  d = 3072 [27]   154 / 158 / 160 / 165    one wave with 8 rows
+  //   n = 12, K = 100, d = 3072 [27]   228 / 224 / 233 / 237    with 4
+  //   n = 8,  K = 128, d = 4096 [12]    71 /  66 /  64 /  65    with 2
+  //   n = 16, K = 250, d = 2048 [41]    73 /  70 /  69 /  74    with 2
+  //   n = 8,  K = 200, d = 4096 [12]    83 /   - /  73 /  72    with 1
+  //   n = 32, K = 240, d = 4096 [95]   171 /   - / 164 / 170    with 1: two rows at least
+  const int64_t P4 = a.P / 4, wave = (int64_t)sm_count * 8;
+  int y = 8;
+  while (y > 2 && (P4 + 256 / y - 1) / (256 / y) > wave) y /= 2;
+  int64_t blocks = (P4 + 256 / y - 1) / (256 / y);
+  blocks = blocks > wave ? wave : blocks < 1 ? 1 : blocks;
+  auto kern = cm ? (y == 8 ? decode_kernel<true, 8> : y == 4 ? decode_kernel<true, 4> : decode_kernel<true, 2>)
+                 : (y == 8 ? decode_kernel<false, 8> : y == 4 ? decode_kernel<false, 4> : decode_kernel<false, 2>);
+  return launch_maybe_pdl(pdl, kern, dim3((unsigned)blocks), dim3(256), st, a, cm ? *cm : CommitArgs{});
 }
 
 // ---------------------------------------------------------------------------

@@ -292,39 +292,39 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
   }
 }
 
-// Decode + SGD of kDecX float4 columns (chunk q), their terms split over kDecY
-// thread rows (for large P, many CTAs).  Must be called by exactly
-// kDecX * kDecY threads, all of which pass every bar().  red: [2 kDecY][kDecX].
+// Decode + SGD of 256 / kY float4 columns (chunk q), their terms split over kY
+// thread rows (for large P, many CTAs).  Must be called by exactly 256 threads,
+// all of which pass every bar().
 // Steady steps: each thread row sums its share of the refreshed slot's stores
 // (the new U[o_t]) and, with their coefficients, of the other slot totals and
 // the deviating stores' slots, all loads of a column in flight over the rows;
 // one exchange.  (One slot after the other, with two barriers each, a step of
-// 12 x 4096 x 3072, K = 100 spent 21 us here, now 16.)
-constexpr int kDecX = 32;
-constexpr int kDecY = 8;
-
-template <class Bar>
-__device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (*red)[kDecX], int tid, int64_t q,
+// 12 x 4096 x 3072, K = 100 spent 21 us here, now 13; beta is read with the
+// terms, not after them: 1 to 2 us of a step.)
+template <int kY, class Bar>
+__device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (*red)[256 / kY], int tid, int64_t q,
                              Bar bar) {
-  const int x = tid % kDecX, y = tid / kDecX;
+  constexpr int kX = 256 / kY;
+  const int x = tid % kX, y = tid / kX;
   const int64_t P4 = a.P / 4;
   const int c = a.c;
   const float B = pl.B;
   const int ndev = pl.ndev;
   const float4* store = reinterpret_cast<const float4*>(a.store);
   float4* U = reinterpret_cast<float4*>(a.U);
-  const int64_t p = q * kDecX + x;
+  const int64_t p = q * kX + x;
   const bool inb = p < P4;
   if (a.slot >= 0) {
-    float4 un = f4zero(), rest = f4zero();
+    float4 un = f4zero(), rest = f4zero(), w = f4zero();
     if (inb) {
+      if (y == 0) w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       if (!a.u_ready) {
         const float4* s0 = store + (int64_t)a.slot * P4 + p;
-        for (int r0 = y; r0 < a.owners; r0 += 4 * kDecY) {
+        for (int r0 = y; r0 < a.owners; r0 += 4 * kY) {
           float4 v[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            v[j] = r0 + j * kDecY < a.owners ? __ldcg(s0 + (int64_t)(r0 + j * kDecY) * c * P4) : f4zero();
+            v[j] = r0 + j * kY < a.owners ? __ldcg(s0 + (int64_t)(r0 + j * kY) * c * P4) : f4zero();
 #pragma unroll
           for (int j = 0; j < 4; ++j) un = f4add(un, v[j]);
         }
@@ -333,12 +333,12 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
       }
       // term t: slot total t (t < c, t != o_t), then slot o of deviating store d
       const int nt = c + ndev * c;
-      for (int t0 = y; t0 < nt; t0 += 4 * kDecY) {
+      for (int t0 = y; t0 < nt; t0 += 4 * kY) {
         float4 v[4];
         float f[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int t = t0 + j * kDecY;
+          const int t = t0 + j * kY;
           v[j] = f4zero();
           f[j] = B;
           if (t < c) {
@@ -354,17 +354,16 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
       }
     }
     red[y][x] = un;
-    red[kDecY + y][x] = rest;
+    red[kY + y][x] = rest;
     bar();
     if (y == 0 && inb) {
 #pragma unroll
-      for (int j = 1; j < kDecY; ++j) {
+      for (int j = 1; j < kY; ++j) {
         un = f4add(un, red[j][x]);
-        rest = f4add(rest, red[kDecY + j][x]);
+        rest = f4add(rest, red[kY + j][x]);
       }
       if (!a.u_ready) U[(int64_t)a.slot * P4 + p] = un;
       const float4 g = f4fma(B, un, rest);
-      float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
       w = f4fma(-a.lr, g, w);
       store_outputs_any(a, p, g, w);
     }
@@ -375,13 +374,13 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
   for (int o = 0; o < c; ++o) {
     float4 part = f4zero();
     if (inb)
-      for (int r = y; r < a.owners; r += kDecY) part = f4add(part, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
+      for (int r = y; r < a.owners; r += kY) part = f4add(part, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
     red[y][x] = part;
     bar();
     if (y == 0) {
       float4 u = red[0][x];
 #pragma unroll
-      for (int j = 1; j < kDecY; ++j) u = f4add(u, red[j][x]);
+      for (int j = 1; j < kY; ++j) u = f4add(u, red[j][x]);
       if (inb) U[(int64_t)o * P4 + p] = u;
       V = f4add(V, u);
     }
@@ -389,7 +388,7 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
   }
   float4 dv = f4zero();
   if (inb)
-    for (int qq = y; qq < ndev; qq += kDecY) {
+    for (int qq = y; qq < ndev; qq += kY) {
       const int r = pl.dev[qq];
       float4 Cr = f4zero();
       for (int o = 0; o < c; ++o) Cr = f4add(Cr, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
@@ -400,7 +399,7 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
   if (y == 0 && inb) {
     float4 D = red[0][x];
 #pragma unroll
-    for (int j = 1; j < kDecY; ++j) D = f4add(D, red[j][x]);
+    for (int j = 1; j < kY; ++j) D = f4add(D, red[j][x]);
     const float4 g = f4fma(B, V, D);
     float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
