@@ -130,7 +130,7 @@ def kernel_label(w: W.Workload, single: bool, dom: int) -> str:
             return "softmax_rows_kernel (16-row tiles split by features over CTA pairs, one pass over X; whole step)"
         return "softmax_smallk_kernel (8-CTA clusters, one pass over X)"
     if w.loss == "softmax":
-        return "CUDA-core softmax gradient kernels"
+        return "split_gemm_kernel (tcgen05, operands in bf16 parts)" if w.K <= 128 else "CUDA-core softmax gradient kernels"
     return "grad_rows kernel with fused commit+decode (whole step)" if single else "grad_rows kernel"
 
 

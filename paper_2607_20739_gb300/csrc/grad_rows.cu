@@ -54,7 +54,7 @@ StageCfg stage_cfg(int variant, int64_t ld, int tail) {
 //   nc = 32   G = 8, R = 4 / R = 2          fp32 75.8 / 82.4   bf16 72.6 / 97.1
 //   nc = 64   G = 8, R = 2 / R = 1          fp32 66.9 / 74.3   bf16 98.0 / 124.4
 // Short rows take R = 4 where R = 8 would leave SMs without a batch for every
-// warp (fr4_logistic_d64's shape).
+// warp (4 partitions of 256 x 64).
 int grad_rows_variant(int dtype, int64_t d, int64_t rows_per_sm, int64_t* ld_out) {
   if (d > max_features(dtype)) return -1;
   const bool bf16 = dtype == PGC_BF16;

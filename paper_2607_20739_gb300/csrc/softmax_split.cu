@@ -24,8 +24,8 @@
 // alternating with a second one where tensor memory has room.
 //
 // Measured, us per step, before (three CUDA-core kernels) and with this file:
-// 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 227; 8 of 4096 x 784
-// fp32, 10 classes: 915 -> 64.  X is read once per kernel (twice per step).  The
+// 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 222; 8 of 4096 x 784
+// fp32, 10 classes: 915 -> 60.  X is read once per kernel (twice per step).  The
 // instructions of the single-thread roles bound an earlier form (282 and 102,
 // with ring positions divided out and descriptors rebuilt for every MMA).
 //
@@ -52,7 +52,7 @@
 // tile's blocks); every row's max and sum of exp per block go to memory and a
 // small kernel combines them.  Before, the tiled CUDA-core logits
 // went through memory, and one more kernel reduced them: a step with its loss on
-// 8 partitions of about 600 x 1500 bf16, 300 classes, took 473 us; now 144
+// 8 partitions of about 600 x 1500 bf16, 300 classes, took 473 us; now 140
 // (184 with the class blocks of a tile one after the other in one cluster: 20
 // of 76 clusters busy).
 //

@@ -242,6 +242,7 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
   const bool small = a.owners <= kMaxO && c <= kMaxC && ndev <= kMaxD && a.slot >= 0 && !a.u_ready;
   for (int64_t p = q0 + tid; p < q1; p += nthr) {
     float4 V = f4zero(), D = f4zero();
+    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     if (small) {
       float4 u[kMaxO], o4[kMaxC], dv[kMaxD][kMaxC];
 #pragma unroll
@@ -286,7 +287,6 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
       }
     }
     const float4 g = f4fma(B, V, D);
-    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
     store_outputs<kUser>(a, p, g, w);
   }
@@ -299,8 +299,8 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
 // (the new U[o_t]) and, with their coefficients, of the other slot totals and
 // the deviating stores' slots, all loads of a column in flight over the rows;
 // one exchange.  (One slot after the other, with two barriers each, a step of
-// 12 x 4096 x 3072, K = 100 spent 21 us here, now 13; beta is read with the
-// terms, not after them: 1 to 2 us of a step.)
+// 12 x 4096 x 3072, K = 100 spent 21 us here, 16 with one exchange.)  beta is read
+// with the terms, not after them: 1 to 2 us of a step.
 template <int kY, class Bar>
 __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (*red)[256 / kY], int tid, int64_t q,
                              Bar bar) {
