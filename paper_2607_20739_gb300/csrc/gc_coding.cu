@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(256) gc_decode_kernel(DecodeArgs a, const floa
   const int64_t P4 = a.P / 4;
   const float4* store = reinterpret_cast<const float4*>(a.store);
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P4; p += (int64_t)gridDim.x * blockDim.x) {
-    float4 g = f4zero(), w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
+    float4 g = f4zero();
     for (int j0 = 0; j0 < cnt; j0 += 16) {
       float4 v[16];
 #pragma unroll
@@ -278,6 +278,7 @@ __global__ void __launch_bounds__(256) gc_decode_kernel(DecodeArgs a, const floa
       for (int u = 0; u < 16; ++u)
         if (j0 + u < cnt) g = f4fma(qw[j0 + u], v[u], g);
     }
+    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
     store_outputs_any(a, p, g, w);
   }

@@ -242,7 +242,11 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
   const bool small = a.owners <= kMaxO && c <= kMaxC && ndev <= kMaxD && a.slot >= 0 && !a.u_ready;
   for (int64_t p = q0 + tid; p < q1; p += nthr) {
     float4 V = f4zero(), D = f4zero();
-    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
+    // in the streaming kernel's tail beta is read with the terms (4 x 256 x 64: 9.8
+    // us per step after them, 9.5 with them); the few-class kernel has no registers
+    // for it (32 x 4096 x 3072: 56.8 after, 58.2 with)
+    constexpr bool kEarly = kUser == kUserPrefix;
+    float4 w = kEarly ? __ldcg(reinterpret_cast<const float4*>(a.w) + p) : f4zero();
     if (small) {
       float4 u[kMaxO], o4[kMaxC], dv[kMaxD][kMaxC];
 #pragma unroll
@@ -287,6 +291,7 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
       }
     }
     const float4 g = f4fma(B, V, D);
+    if (!kEarly) w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
     store_outputs<kUser>(a, p, g, w);
   }
