@@ -75,7 +75,7 @@ cudaError_t launch_commit(const CommitArgs& a, cudaStream_t st, bool pdl) {
 // reads only that column of the stores, so a CTA barrier is enough): thread
 // row y sums the items of partitions y, y + kY, ..., in item order.  One
 // launch instead of two.
-template <bool kCommit, int kY>
+template <bool kCommit, int kY, bool kAll>
 __global__ void __launch_bounds__(256) decode_kernel(DecodeArgs a, CommitArgs cm) {
   constexpr int kX = 256 / kY;
   __shared__ DecodePlan pl;
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) decode_kernel(DecodeArgs a, CommitArgs cm
       }
       __syncthreads();
     }
-    decode_chunk<kY>(a, pl, red, (int)threadIdx.x, q, bar);
+    decode_chunk<kY, kAll>(a, pl, red, (int)threadIdx.x, q, bar);
   }
 }
 
@@ -202,6 +202,11 @@ constexpr int64_t kWideDecodeMinP4 = 1 << 18;
 
 bool decode_commits(int64_t P) { return P / 4 < kWideDecodeMinP4; }
 
+template <bool kCommit, bool kAll>
+static auto decode_instance(int y) {
+  return y == 8 ? decode_kernel<kCommit, 8, kAll> : y == 4 ? decode_kernel<kCommit, 4, kAll> : decode_kernel<kCommit, 2, kAll>;
+}
+
 cudaError_t launch_decode(const DecodeArgs& a, const CommitArgs* cm, cudaStream_t st, bool pdl, int sm_count) {
   if (a.n > kMaxWorkers || a.owners > kMaxWorkers) return cudaErrorInvalidValue;
   if (a.P / 4 >= kWideDecodeMinP4) {
@@ -224,8 +229,10 @@ cudaError_t launch_decode(const DecodeArgs& a, const CommitArgs* cm, cudaStream_
   while (y > 2 && (P4 + 256 / y - 1) / (256 / y) > wave) y /= 2;
   int64_t blocks = (P4 + 256 / y - 1) / (256 / y);
   blocks = blocks > wave ? wave : blocks < 1 ? 1 : blocks;
-  auto kern = cm ? (y == 8 ? decode_kernel<true, 8> : y == 4 ? decode_kernel<true, 4> : decode_kernel<true, 2>)
-                 : (y == 8 ? decode_kernel<false, 8> : y == 4 ? decode_kernel<false, 4> : decode_kernel<false, 2>);
+  // the refresh of every slot has instances of its own: its registers are not the steady step's
+  const bool all = a.slot < 0;
+  auto kern = cm ? (all ? decode_instance<true, true>(y) : decode_instance<true, false>(y))
+                 : (all ? decode_instance<false, true>(y) : decode_instance<false, false>(y));
   return launch_maybe_pdl(pdl, kern, dim3((unsigned)blocks), dim3(256), st, a, cm ? *cm : CommitArgs{});
 }
 

@@ -299,14 +299,15 @@ __device__ __forceinline__ void decode_columns(const DecodeArgs& a, const Decode
 
 // Decode + SGD of 256 / kY float4 columns (chunk q), their terms split over kY
 // thread rows (for large P, many CTAs).  Must be called by exactly 256 threads,
-// all of which pass every bar().
+// all of which pass every bar().  red: [2 kY][256 / kY].  kAll: every slot is
+// refreshed (a.slot < 0), else the one slot.
 // Steady steps: each thread row sums its share of the refreshed slot's stores
 // (the new U[o_t]) and, with their coefficients, of the other slot totals and
 // the deviating stores' slots, all loads of a column in flight over the rows;
 // one exchange.  (One slot after the other, with two barriers each, a step of
 // 12 x 4096 x 3072, K = 100 spent 21 us here, 16 with one exchange.)  beta is read
 // with the terms, not after them: 1 to 2 us of a step.
-template <int kY, class Bar>
+template <int kY, bool kAll, class Bar>
 __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (*red)[256 / kY], int tid, int64_t q,
                              Bar bar) {
   constexpr int kX = 256 / kY;
@@ -319,7 +320,7 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
   float4* U = reinterpret_cast<float4*>(a.U);
   const int64_t p = q * kX + x;
   const bool inb = p < P4;
-  if (a.slot >= 0) {
+  if constexpr (!kAll) {
     float4 un = f4zero(), rest = f4zero(), w = f4zero();
     if (inb) {
       if (y == 0) w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
@@ -375,19 +376,33 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
     bar();
     return;
   }
-  float4 V = f4zero();
-  for (int o = 0; o < c; ++o) {
-    float4 part = f4zero();
+  // warm-up, gradient coding: two slots per exchange (one: 26.1 us per step at
+  // 16 x 1000 x 1000, K = 10; two: 24.8; four: 24.7, but their shared memory kept CTAs from
+  // starting beside the kernel before)
+  float4 V = f4zero(), w = f4zero();
+  if (inb && y == 0) w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
+  for (int o0 = 0; o0 < c; o0 += 2) {
+    float4 part[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) part[j] = f4zero();
     if (inb)
-      for (int r = y; r < a.owners; r += kY) part = f4add(part, __ldcg(store + ((int64_t)r * c + o) * P4 + p));
-    red[y][x] = part;
+      for (int r = y; r < a.owners; r += kY)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (o0 + j < c) part[j] = f4add(part[j], __ldcg(store + ((int64_t)r * c + o0 + j) * P4 + p));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) red[j * kY + y][x] = part[j];
     bar();
     if (y == 0) {
-      float4 u = red[0][x];
 #pragma unroll
-      for (int j = 1; j < kY; ++j) u = f4add(u, red[j][x]);
-      if (inb) U[(int64_t)o * P4 + p] = u;
-      V = f4add(V, u);
+      for (int j = 0; j < 2; ++j) {
+        if (o0 + j >= c) break;
+        float4 u = red[j * kY][x];
+#pragma unroll
+        for (int i = 1; i < kY; ++i) u = f4add(u, red[j * kY + i][x]);
+        if (inb) U[(int64_t)(o0 + j) * P4 + p] = u;
+        V = f4add(V, u);
+      }
     }
     bar();
   }
@@ -406,7 +421,6 @@ __device__ void decode_chunk(const DecodeArgs& a, const DecodePlan& pl, float4 (
 #pragma unroll
     for (int j = 1; j < kY; ++j) D = f4add(D, red[j][x]);
     const float4 g = f4fma(B, V, D);
-    float4 w = __ldcg(reinterpret_cast<const float4*>(a.w) + p);
     w = f4fma(-a.lr, g, w);
     store_outputs_any(a, p, g, w);
   }
