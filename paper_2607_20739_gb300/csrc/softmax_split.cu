@@ -53,8 +53,8 @@
 // small kernel combines them.  Before, the tiled CUDA-core logits
 // went through memory, and one more kernel reduced them: a step with its loss on
 // 8 partitions of about 600 x 1500 bf16, 300 classes, took 473 us; now 140
-// (184 with the class blocks of a tile one after the other in one cluster: 20
-// of 76 clusters busy).
+// (184 against 144 with the class blocks of a tile one after the other in one
+// cluster: 20 of 76 clusters busy).
 //
 // Every wait is bounded; on a failure the kernel flags the status word, all
 // roles wind down, and TMEM is released after the MMAs issued so far.
