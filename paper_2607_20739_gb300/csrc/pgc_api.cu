@@ -252,12 +252,15 @@ void add_item(pgc_ctx* ctx, Phase& ph, int e, int64_t r0, int64_t rows) {
 // 16384: 292, 368, 409 us per step against 277, 317, 350 with runs across
 // partitions; fp32, d = 3001: 311 against 300), and pays for fp32 rows from
 // 16 KB on, which 128 SMs stream at the HBM rate with fewer streams (d = 8192: 283
-// against 297; 64 x 2048 x 16384: 1225 against 1264).
+// against 297; 64 x 2048 x 16384: 1225 against 1264).  With more partitions than
+// SMs such runs would not reach the last ones: there a run always crosses
+// (153 partitions of 200 x 4096 fp32: 81 us per step, 115 with items taken
+// dynamically; 200 of 40 x 8192: 59, 69; 1024 of 8 x 16384: 239, 241).
 void build_row_ranges(pgc_ctx* ctx, Phase& ph) {
   const int nE = (int)ph.parts.size();
   const int64_t least = grad_rows_min_item(ctx->variant);
   const int64_t h = std::max<int64_t>(1, 49152 / (ctx->ld * (int64_t)ctx->esize));
-  const bool cross = ctx->dtype == PGC_BF16 || ctx->ld * (int64_t)ctx->esize < 16384;
+  const bool cross = ctx->dtype == PGC_BF16 || ctx->ld * (int64_t)ctx->esize < 16384 || nE > ctx->sm_count;
   std::vector<int64_t> run;                 // e, first row, rows of every item; -1: next CTA
   auto fill = [&](int64_t C) {
     run.clear();
@@ -837,7 +840,14 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   ctx->phases.resize(1 + ctx->c);
   build_phase(ctx, ctx->phases[0], -1);
   for (int o = 0; o < ctx->c; ++o) build_phase(ctx, ctx->phases[1 + o], o);
-  for (auto& ph : ctx->phases) ph.tail = ctx->loss == PGC_SOFTMAX ? 0 : ctx->tail_mode;
+  for (auto& ph : ctx->phases) {
+    ph.tail = ctx->loss == PGC_SOFTMAX ? 0 : ctx->tail_mode;
+    if (ctx->loss == PGC_SOFTMAX) continue;
+    // a row without an item would be left out of the gradient without a word
+    int64_t covered = 0;
+    for (const WorkItem& it : ph.items) covered += it.rows;
+    if (covered != ph.z_total) { delete ctx; return PGC_ENOTSUP; }
+  }
   size_t max_partials = 0;
   int64_t max_z = 0;
   for (auto& ph : ctx->phases) {
