@@ -354,6 +354,7 @@ int pgc_timing_read(pgc_ctx *ctx, double *ms, int64_t *launches, int64_t *steps_
  *
  *   X     : device [m][d] features (PGC_F32, or PGC_BF16 bits), 16-byte aligned
  *   y     : device [m] float32 labels;  w: device [d] float32 parameters
+ *           (both 4-byte aligned)
  *   g_out : device [d] float32, 16-byte aligned (written)
  *   stream: cudaStream_t to run on; the call waits for it before returning.
  *

@@ -46,7 +46,8 @@ void* g_scratch_ptr[kMaxDevices] = {};
 
 // Scratch layout (bytes): [0,4) status word; [16,24) e_item0[2];
 // [32,36) e_scale[1]; [48,52) e_dest[1]; [256, 256 + items) work items;
-// then the per-CTA partial sums, 256-byte aligned.
+// the labels; the per-CTA partial sums, 256-byte aligned; w, if it had to be
+// copied.
 constexpr size_t kOffStatus = 0, kOffItem0 = 16, kOffScale = 32, kOffDest = 48, kOffItems = 256;
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -115,7 +116,14 @@ extern "C" int pgc_gradient_noalloc(int32_t loss, int32_t dtype, int64_t m, int6
   // and may read 12 bytes past the last one, so it reads a padded copy here
   const size_t off_labels = align256(kOffItems + (size_t)G * sizeof(pgc::WorkItem));
   const size_t off_partials = align256(off_labels + (size_t)m * sizeof(float) + 16);
-  if (off_partials + (size_t)G * (size_t)ld * sizeof(float) > kScratchBytes) return PGC_ESCRATCH;
+  const size_t row_bytes = (size_t)ld * sizeof(float);
+  if (off_partials + (size_t)G * row_bytes > kScratchBytes) return PGC_ESCRATCH;
+  // it also reads w in 16-byte pieces: a w that lies elsewhere is copied behind
+  // the partials, in the place of the last one where the scratch is full
+  const bool copy_w = reinterpret_cast<uintptr_t>(w) % 16 != 0;
+  if (copy_w && G > 1 && off_partials + (size_t)(G + 1) * row_bytes > kScratchBytes) --G;
+  const size_t off_w = off_partials + (size_t)G * row_bytes;
+  if (copy_w && off_w + row_bytes > kScratchBytes) return PGC_ESCRATCH;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   noalloc_fill_tables<<<(unsigned)((G + 255) / 256), 256, 0, st>>>(scratch, (int)G, m);
@@ -123,6 +131,10 @@ extern "C" int pgc_gradient_noalloc(int32_t loss, int32_t dtype, int64_t m, int6
   if (cudaMemcpyAsync(scratch + off_labels, y, (size_t)m * sizeof(float), cudaMemcpyDeviceToDevice, st) !=
       cudaSuccess)
     return PGC_ECUDA;
+  if (copy_w) {
+    if (cudaMemcpyAsync(scratch + off_w, w, row_bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return PGC_ECUDA;
+    w = reinterpret_cast<const float*>(scratch + off_w);
+  }
 
   pgc::GradRowsArgs g;
   g.loss = loss; g.dtype = dtype; g.d = d; g.ld = ld; g.X = X;

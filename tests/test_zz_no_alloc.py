@@ -87,3 +87,30 @@ def test_noalloc_rejects_what_it_cannot_hold(libpgc, cuda):
                                        C.c_void_p(g.data_ptr()), None)
     assert big == lib.ESCRATCH
     assert b"scratch" in lib.lib.pgc_strerror(lib.ESCRATCH)
+
+
+@pytest.mark.parametrize("dtype,d,m", [("f32", 32, 200), ("f32", 1024, 301), ("f32", 16384, 20), ("bf16", 64, 500), ("bf16", 2048, 77),
+                                       ("bf16", 32768, 127)])
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_noalloc_takes_w_at_any_float(libpgc, cuda, dtype, d, m, off):
+    """X and g_out are documented as 16-byte aligned, y and w are not: a slice
+    of a larger parameter vector gives the same gradient, bit for bit.  (The
+    last case fills the scratch with partial sums: w takes the place of one,
+    so the rows are cut elsewhere, and only the bound holds.)"""
+    torch = cuda
+    code = libpgc.F32 if dtype == "f32" else libpgc.BF16
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    X = torch.randn((m, d), generator=gen, device="cuda")
+    X = X if dtype == "f32" else X.to(torch.bfloat16)
+    y, flat = torch.rand(m + 4, generator=gen, device="cuda"), torch.randn(d + 4, generator=gen, device="cuda") / d ** 0.5
+    torch.cuda.synchronize()
+    want, got = (torch.full((d,), float("nan"), device="cuda") for _ in range(2))
+    for out, yy, ww in ((want, y[off:off + m].clone(), flat[off:off + d].clone()), (got, y[off:off + m], flat[off:off + d])):
+        torch.cuda.synchronize()
+        assert ww.data_ptr() % 16 == (0 if out is want else 4 * off)
+        assert _noalloc(libpgc, libpgc.LSQ, code, X, yy, ww, out) == libpgc.OK
+    if d != 32768:
+        torch.testing.assert_close(got, want, rtol=0, atol=0)
+    x = X.double()
+    exact = (x @ flat[off:off + d].double() - y[off:off + m].double()) @ x / m
+    assert float((got.double() - exact).abs().max() / exact.abs().max()) <= TOL
