@@ -183,8 +183,9 @@ int pgc_load_partitions(pgc_ctx *ctx, const void *const *X, const void *const *y
  *                    call returns without waiting for the GPU; 0: host
  *                    pointers, the call waits until they hold the results
  *                    (pinned host buffers mapped into the device's address
- *                    space are written by the decode kernel itself; others
- *                    are filled by copies after it).
+ *                    space are written by the decode kernel itself, unless
+ *                    they are large and their rows of d floats do not all
+ *                    start on 16 bytes; others are filled by copies after it).
  *   info           : may be NULL; receives t, o_t and the schedule indices.
  * Step 0 is the warm-up: every worker evaluates all c of its partitions at
  * beta^(0).  From step 1 on, worker W_i evaluates only the partition in its

@@ -611,6 +611,9 @@ void free_all(pgc_ctx* ctx) {
   ctx->loss_h = nullptr;
 }
 
+// Floats of an output up to which the decode writes host rows of any alignment itself.
+constexpr int64_t kHostFloats = 330000;
+
 // Device address of a pinned host buffer mapped into the current device's
 // address space, or nullptr (pageable memory, or not addressable).
 void* mapped_host(const void* p) {
@@ -1216,7 +1219,12 @@ int pgc_step(pgc_ctx* ctx, const uint8_t* mask, float* grad_out, float* w_out, i
   }
   const uintptr_t addr = reinterpret_cast<uintptr_t>(g_dev) | reinterpret_cast<uintptr_t>(w_dev);
   const bool same = (ctx->K == 1 || ctx->ld == ctx->d) && addr % 16 == 0;
-  const bool direct = (!grad_out || g_dev) && (!w_out || w_dev) && (same || (ctx->K > 1 && addr % 4 == 0));
+  // Host rows that do not all start on 16 bytes are written float by float, a
+  // transfer over the link each: faster than copies only up to about 330,000 floats
+  // (K = 200: d = 1501 81 us per step, 84 with copies; 1701 94, 86; K = 1000:
+  // d = 301 73, 79; 401 88, 80; 3001 540, 233).
+  const bool by_float = !outputs_on_device && (ctx->d % 4 != 0 || addr % 16 != 0) && ctx->K * ctx->d > kHostFloats;
+  const bool direct = (!grad_out || g_dev) && (!w_out || w_dev) && (same || (ctx->K > 1 && addr % 4 == 0 && !by_float));
   if (direct) {
     dc.g_user = g_dev;
     dc.w_user = w_dev;

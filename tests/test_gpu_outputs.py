@@ -69,3 +69,45 @@ def test_outputs(libpgc, cuda, name):
     np.testing.assert_array_equal(only.cpu().numpy(), g.weights().reshape(-1))
     g.close()
     ref.close()
+
+
+@pytest.mark.parametrize("K,d,off", [(130, 2538, 0), (130, 2539, 0), (130, 2540, 1), (130, 2540, 0), (1000, 333, 0)])
+def test_host_rows_around_the_size_that_copies_take(libpgc, cuda, K, d, off):
+    """Pinned rows that start off 16 bytes: written by the decode up to 330,000
+    floats, copied from there on."""
+    torch = cuda
+    w = WL["cr_n128_softmax_k1000"].replace(n=3, s=1, K=K, d=d, m=20)
+    Xs, ys, masks = generate(w, 2)
+    g, size = make_gpu(libpgc, w, Xs, ys), K * d
+    for t in range(2):
+        gb, wb = (torch.full((size + off + 8,), 7.0).pin_memory() for _ in range(2))
+        before = g.weights().reshape(-1)
+        g.step(masks[t], gb[off:off + size], wb[off:off + size])
+        np.testing.assert_array_equal(wb[off:off + size].numpy(), g.weights().reshape(-1))
+        moved = before - np.float32(w.lr) * gb[off:off + size].numpy()
+        assert np.abs(moved - g.weights().reshape(-1)).max() <= 1e-6 * np.abs(moved).max()   # one rounding more than the fused update
+        for b in (gb, wb):
+            assert (b[:off] == 7.0).all() and (b[off + size:] == 7.0).all()
+    g.close()
+
+
+def test_large_unaligned_host_rows_do_not_hold_up_the_decode(libpgc, cuda):
+    """Float by float over the link, three million floats took the decode
+    fifteen times as long as on the device; with copies it takes the same time."""
+    torch = cuda
+    w = WL["cr_n128_softmax_k1000"].replace(n=3, s=1, K=1000, d=3001, m=20)
+    Xs, ys, masks = generate(w, 1)
+    g, ms = make_gpu(libpgc, w, Xs, ys), {}
+    for where in ("device", "host"):
+        make = (lambda: torch.zeros(w.K * w.d, device="cuda")) if where == "device" else \
+            (lambda: torch.zeros(w.K * w.d).pin_memory())
+        a, b = make(), make()
+        for _ in range(4):
+            g.step(masks[0], a, b)
+        g.timing(True)
+        for _ in range(10):
+            g.step(masks[0], a, b)
+        ms[where] = g.timing_read()["ms"][libpgc.KERNEL_GROUPS.index("decode")]
+        g.timing(False)
+    g.close()
+    assert ms["host"] < 4 * ms["device"], ms
