@@ -542,9 +542,10 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmB, SplitArgs p) {
             if (c < nc) m = fmaxf(m, z[c]);
             if (c < nc && c == lab) p.row_lab[row] = z[c];
           }
+          const float base = m == -INFINITY ? 0.f : m;       // every class of the block masked: sum 0 (NaN logits still count)
 #pragma unroll
           for (int c = 0; c < NCH * 32; ++c)
-            if (c < nc) sum += expf(z[c] - m);
+            if (c < nc) sum += expf(z[c] - base);
           p.row_stats[(int64_t)u.e * p.rows + row] = make_float2(m, sum);
         }
       } else if constexpr (!kGrad) {

@@ -142,10 +142,20 @@ __device__ __forceinline__ void write_coeffs_warp(const DecodeArgs& a, int lane)
 
 // Four parameters (float4 column i) as three bf16 parts each, w = w1 + w2 + w3
 // up to 2^-27 |w| (round to nearest); part j of the array starts at j * stride.
+// Beyond bf16's largest value (3.39e38; a class masked by fp32's lowest value or by
+// -infinity) a part is that value, not the infinity it would round to, whose
+// remainder has the other sign or is NaN; an infinity becomes three of them.
+constexpr float kBf16Max = 3.3895313892515355e38f;           // (2 - 2^-7) 2^127
+__device__ __forceinline__ float bf16_range(float v) {
+  return fabsf(v) > kBf16Max ? copysignf(kBf16Max, v) : v;   // NaN stays
+}
 __device__ __forceinline__ void store_split4(uint16_t* dst, int64_t stride, int64_t i, float4 v) {
+  const bool beyond = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))) > kBf16Max;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    float4 r = v;
+    if (beyond) r = make_float4(bf16_range(v.x), bf16_range(v.y), bf16_range(v.z), bf16_range(v.w));
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(r.x, r.y), hi = __floats2bfloat162_rn(r.z, r.w);
     uint2 pk;
     pk.x = *reinterpret_cast<const uint32_t*>(&lo);
     pk.y = *reinterpret_cast<const uint32_t*>(&hi);
