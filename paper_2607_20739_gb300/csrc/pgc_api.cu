@@ -697,12 +697,18 @@ int pgc_create(pgc_ctx** out, int32_t n, int32_t s, int32_t scheme, int32_t loss
 
 namespace {
 
-// pgc_create_mode; *split: in, whether the single-precision tensor-core
-// softmax path may be taken; out, whether it was.
+// What a context can do without where memory is short: in, whether it may be
+// used; out, whether it was.
+struct Optional {
+  bool split = true;   // the single-precision tensor-core softmax path (its residuals)
+  bool loss = true;    // the tensor-core loss (parts of W, row statistics)
+};
+
+// pgc_create_mode with the optional parts it is allowed.
 int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t scheme, int32_t loss, int32_t dtype,
-                   int64_t d, int64_t K, const int64_t* rows, float lr, const float* w0, void* stream, bool* split) {
-  const bool allow_split = *split;
-  *split = false;
+                   int64_t d, int64_t K, const int64_t* rows, float lr, const float* w0, void* stream, Optional* opt) {
+  const bool allow_split = opt->split, allow_loss = opt->loss;
+  *opt = {false, false};
   int rc = check_nsc(scheme, n, s);
   if (rc) return rc;
   if (mode != PGC_MODE_PGC && mode != PGC_MODE_IS_SGD && mode != PGC_MODE_GC && mode != PGC_MODE_NAIVE_CR)
@@ -812,7 +818,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     // (PGC_NO_SPLIT=1 keeps the CUDA-core kernels)
     if (!ctx->tc && !ctx->smallk && allow_split && K <= kSplitMaxClasses && !no_split) {
       ctx->sp_nc = std::min(split_max_clusters(kSplitLogits, dtype, K), split_max_clusters(kSplitGrad, dtype, K));
-      ctx->split = *split = ctx->sp_nc > 0;
+      ctx->split = opt->split = ctx->sp_nc > 0;
       ctx->sp_Kp = split_kp(K);
       ctx->sp_C3 = split_cols(ctx->sp_Kp);
       std::vector<int64_t> steady;   // rows of the partitions a steady step evaluates
@@ -932,7 +938,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
   PGC_ALLOC(ctx->partials, max_partials * sizeof(float));
   int64_t max_zpad = 0;
   for (auto& ph : ctx->phases) max_zpad = std::max(max_zpad, ph.zpad_total);
-  if (loss == PGC_SOFTMAX && !no_split && ctx->total_rows < (int64_t(1) << 31) - 2 * kSplitTile) {
+  if (loss == PGC_SOFTMAX && allow_loss && !no_split && ctx->total_rows < (int64_t(1) << 31) - 2 * kSplitTile) {
     // the loss on the tensor cores, if the parts of W fit
     const int nc = split_max_clusters(kSplitLoss, dtype, std::min(K, kSplitMaxClasses));
     ctx->lw_Kp = split_kp(std::min(K, kSplitMaxClasses));
@@ -943,10 +949,13 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     if (nc > 0 && (ctx->split || cudaMalloc((void**)&ctx->lw, parts) == cudaSuccess) &&
         cudaMalloc((void**)&ctx->row_stats, rows_b) == cudaSuccess) {
       ctx->lw_nc = nc;
+      opt->loss = true;
       ctx->row_lab = reinterpret_cast<float*>(ctx->row_stats + ctx->total_rows * ctx->lw_ncb);
       PGC_ALLOC(ctx->tmXl, 128);
     } else {
       cudaGetLastError();
+      if (ctx->lw && ctx->lw != ctx->wb) cudaFree(ctx->lw);   // nothing uses it alone
+      ctx->lw = nullptr;
     }
   } else if (loss != PGC_SOFTMAX) {
     ctx->loss_nblocks = 8 * ctx->sm_count;
@@ -1135,16 +1144,17 @@ int pgc_create_mode(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t s
                     void* stream) {
   if (!out) return PGC_EINVAL;
   *out = nullptr;
-  bool split = true;
-  int rc = create_context(out, mode, n, s, scheme, loss, dtype, d, K, rows, lr, w0, stream, &split);
-  if (rc == PGC_ENOMEM && split) {
-    // its residual buffer is larger than the CUDA-core kernels': a run that
-    // fits only without it takes them
+  // A run that fits only without the tensor-core loss or the split residuals does
+  // without them (their buffers are larger than those of the kernels they
+  // replace): each attempt gives up one part that the one before it used.
+  Optional use;
+  for (;;) {
+    const int rc = create_context(out, mode, n, s, scheme, loss, dtype, d, K, rows, lr, w0, stream, &use);
+    if (rc != PGC_ENOMEM || (!use.loss && !use.split)) return rc;
     cudaGetLastError();
-    split = false;
-    rc = create_context(out, mode, n, s, scheme, loss, dtype, d, K, rows, lr, w0, stream, &split);
+    if (use.loss) use.loss = false;
+    else use = {false, true};
   }
-  return rc;
 }
 
 int pgc_destroy(pgc_ctx* ctx) {
