@@ -772,6 +772,9 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     //   1 MB    d = 64: 19 / 14   256: 14 / 14   1024: 14 / 17
     // Over these points the choice costs 0.2 % against the better kernel on average
     // (12 % at worst: 25 MB, d = 1250).  Below 2048 rows the two are within 1 us.
+    auto split_clusters = [&] {
+      return std::min(split_max_clusters(kSplitLogits, dtype, K), split_max_clusters(kSplitGrad, dtype, K));
+    };
     bool few_split = false;
     if (!ctx->tc && dtype == PGC_BF16 && K <= 16 && allow_split && !no_split && !std::getenv("PGC_NO_ROWS") &&
         !std::getenv("PGC_NO_ROWS_TAIL")) {
@@ -779,7 +782,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
       const double dd = (double)d;
       const double t_rows = 12.8 + R * (0.826e-3 + 0.139e-6 * dd);
       const double t_split = 12.5 + 0.0043 * dd + R * (0.082e-3 + 0.557e-6 * dd);
-      few_split = R >= 2048 && t_split < t_rows;
+      few_split = R >= 2048 && t_split < t_rows && split_clusters() > 0;
     }
     const char* env2 = std::getenv("PGC_NO_SMALLK");
     const char* env4 = std::getenv("PGC_NO_ROWS");
@@ -817,7 +820,7 @@ int create_context(pgc_ctx** out, int32_t mode, int32_t n, int32_t s, int32_t sc
     // up to 128 classes in single precision: tensor cores on split operands
     // (PGC_NO_SPLIT=1 keeps the CUDA-core kernels)
     if (!ctx->tc && !ctx->smallk && allow_split && K <= kSplitMaxClasses && !no_split) {
-      ctx->sp_nc = std::min(split_max_clusters(kSplitLogits, dtype, K), split_max_clusters(kSplitGrad, dtype, K));
+      ctx->sp_nc = split_clusters();
       ctx->split = opt->split = ctx->sp_nc > 0;
       ctx->sp_Kp = split_kp(K);
       ctx->sp_C3 = split_cols(ctx->sp_Kp);
