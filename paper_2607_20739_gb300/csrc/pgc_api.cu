@@ -1446,7 +1446,7 @@ int pgc_loss(pgc_ctx* ctx, double* loss_out) {
     a.y = static_cast<const int32_t*>(ctx->y); a.status = ctx->status;
     PGC_CK(ctx, launch_split(kSplitLoss, ctx->dtype, ctx->tmWl, a, ctx->lw_nc, ctx->pdl, ctx->stream));
     PGC_CK(ctx, launch_loss_combine(ctx->row_stats, ctx->row_lab, ctx->total_rows, ctx->lw_ncb, ctx->loss_blocks,
-                                    ctx->loss_nblocks, ctx->counters + ctx->n + 3, ctx->loss_out, ctx->stream));
+                                    ctx->loss_nblocks, ctx->counters + ctx->n + 3, ctx->loss_out, ctx->pdl, ctx->stream));
   } else {
     LossArgs a;
     a.loss = ctx->loss; a.dtype = ctx->dtype; a.ld = ctx->ld; a.K = ctx->K; a.rows = ctx->total_rows;

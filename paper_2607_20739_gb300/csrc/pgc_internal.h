@@ -425,7 +425,7 @@ cudaError_t launch_split(int mode, int dtype, const void* tmB, const SplitArgs& 
                          cudaStream_t st);
 // out = mean over the rows of log sum exp - label logit; ticket: a zero word, returned to zero
 cudaError_t launch_loss_combine(const float2* stats, const float* lab, int64_t rows, int ncb, double* blocksum,
-                                int max_blocks, int* ticket, double* out, cudaStream_t st);
+                                int max_blocks, int* ticket, double* out, bool pdl, cudaStream_t st);
 // w [K][ld] -> parts [ceil(K / Kp)][3][Kp][ld] (rows past K are not written)
 cudaError_t launch_split_weights(const float* src, uint16_t* dst, int64_t K, int64_t ld, int Kp, cudaStream_t st);
 // 2-D tensor map [outer][inner], row pitch in bytes, box {box_inner, box_outer}, 128-byte swizzle or none

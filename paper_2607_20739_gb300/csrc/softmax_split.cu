@@ -742,7 +742,7 @@ __global__ void __launch_bounds__(256) loss_combine_kernel(const float2* __restr
 }
 
 cudaError_t launch_loss_combine(const float2* stats, const float* lab, int64_t rows, int ncb, double* blocksum,
-                                int max_blocks, int* ticket, double* out, cudaStream_t st) {
+                                int max_blocks, int* ticket, double* out, bool pdl, cudaStream_t st) {
   int64_t blocks = (rows + 255) / 256;
   if (blocks > max_blocks) blocks = max_blocks;
   cudaLaunchConfig_t cfg = {};
@@ -753,7 +753,7 @@ cudaError_t launch_loss_combine(const float2* stats, const float* lab, int64_t r
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, loss_combine_kernel, stats, lab, rows, ncb, blocksum, ticket, out);
 }
 

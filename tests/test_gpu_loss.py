@@ -50,3 +50,9 @@ def test_softmax_loss_on_cuda_cores(libpgc, cuda, monkeypatch, K):
 @pytest.mark.parametrize("d", [1, 33, 1000, 3001, 5000])
 def test_rows_loss(libpgc, cuda, loss, dtype, d):
     check(libpgc, ROWS.replace(loss=loss, dtype=dtype, d=d, m=(300, 1, 65)))
+
+
+@pytest.mark.parametrize("K", [20, 300])
+def test_softmax_loss_without_dependent_launches(libpgc, cuda, monkeypatch, K):
+    monkeypatch.setenv("PGC_NO_PDL", "1")
+    check(libpgc, SOFTMAX.replace(dtype="bf16", K=K, d=100, m=(300, 1, 65)))
