@@ -70,6 +70,20 @@ def run_gpu(binding, w: W.Workload, Xs, ys, masks, record_loss=True, mode="pgc")
     return g, out
 
 
+def gradient_launches(binding, g, mask) -> int:
+    """Kernels that one more step launches for its gradients.  Two names of
+    paths are shared: "softmax_cc" is the split tensor-core pair (2) and the
+    CUDA-core kernels that stand in for it (3)."""
+    g.timing(True)
+    g.step(mask, info=False)
+    n = g.timing_read()["launches"][binding.KERNEL_GROUPS.index("gradient")]
+    g.timing(False)
+    return n
+
+
+SPLIT_LAUNCHES, CUDA_CORE_LAUNCHES = 2, 3
+
+
 def compare_step(w: W.Workload, t: int, a: dict, b: dict, check_loss=True):
     """One step of a GPU record `a` against the oracle's `b`: schedule, slot,
     FR representatives and the decode support bit-exact, the coefficients to

@@ -12,7 +12,7 @@ import pytest
 
 from paper_2607_20739_gb300 import workloads as W
 
-from parity import compare_runs, generate, rel_err, run_gpu, run_oracle
+from parity import SPLIT_LAUNCHES, compare_runs, generate, gradient_launches, rel_err, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -34,4 +34,5 @@ def test_decode_thread_rows(libpgc, cuda, monkeypatch, K, d, rows):
         compare_runs(w, recs, ora)
         for a, b in zip(recs, ora):
             assert rel_err(a["grad"], b["grad"]) < TOL
+        assert gradient_launches(libpgc, g, masks[0]) == SPLIT_LAUNCHES
         g.close()

@@ -16,7 +16,8 @@ import pytest
 
 from paper_2607_20739_gb300 import workloads as W
 
-from parity import compare_runs, generate, make_gpu, rel_err, run_gpu, run_oracle
+from parity import (CUDA_CORE_LAUNCHES, SPLIT_LAUNCHES, compare_runs, generate, gradient_launches, make_gpu, rel_err,
+                    run_gpu, run_oracle)
 
 pytestmark = pytest.mark.gpu
 
@@ -50,6 +51,7 @@ def test_split_softmax_edges(libpgc, cuda, monkeypatch, dtype, K, d, m):
     compare_runs(w, recs, ora)
     for a, b in zip(recs, ora):
         assert rel_err(a["grad"], b["grad"]) < TOL
+    assert gradient_launches(libpgc, g, masks[0]) == SPLIT_LAUNCHES
     g.close()
 
 
@@ -64,6 +66,7 @@ def test_split_softmax_schemes(libpgc, cuda, scheme, mode, n, s):
         ora = run_oracle(w, Xs, ys, masks, mode=mode)
         for a, b in zip(recs, ora):
             assert rel_err(a["grad"], b["grad"]) < TOL
+        assert gradient_launches(libpgc, g, masks[0]) == SPLIT_LAUNCHES
         g.close()
 
 
@@ -120,6 +123,7 @@ def test_cuda_core_softmax_matches_oracle(libpgc, cuda, monkeypatch, dtype):
     assert g.gradient_path == "softmax_cc"
     for a, b in zip(recs, run_oracle(w, Xs, ys, masks)):
         assert rel_err(a["grad"], b["grad"]) < TOL
+    assert gradient_launches(libpgc, g, masks[0]) == CUDA_CORE_LAUNCHES
     g.close()
 
 
@@ -135,6 +139,23 @@ def test_few_classes_take_the_faster_path(libpgc, cuda, d, m, path, mode):
         g, recs = run_gpu(libpgc, w, Xs, ys, masks)
         compare_runs(w, recs, run_oracle(w, Xs, ys, masks))
     else:
-        g = libpgc.PGC(w.scheme, w.n, w.s, w.loss, w.dtype, w.d, K=w.K, rows=w.rows(), lr=w.lr, mode=mode)
+        from test_gpu_naive_cr import run_and_compare
+        run_and_compare(libpgc, w, 5)                # steps, so that later ones read the parts the weighted decode wrote
+        g = make_gpu(libpgc, w, *generate(w, 1)[:2], mode=mode)
+        g.set_gc_encoding(W.make_gc_draws(w, 5))
+        masks = W.make_masks(w, 1, 7)
     assert g.gradient_path == path
+    assert gradient_launches(libpgc, g, masks[0]) == (SPLIT_LAUNCHES if path == "softmax_cc" else 1)
     g.close()
+
+
+@pytest.mark.parametrize("dtype,K", [("f32", 10), ("bf16", 40)])
+@pytest.mark.parametrize("m", [100, 900])
+@pytest.mark.parametrize("mode", ["naive_cr", "gc"])
+def test_split_softmax_with_the_weighted_decode(libpgc, cuda, dtype, K, m, mode):
+    """GC-CR's decode writes beta's parts anew each step; rows in one unit per
+    partition (100) and in several with partials (900)."""
+    from test_gpu_naive_cr import run_and_compare
+    w = BASE.replace(scheme="CR", n=6, s=2, dtype=dtype, K=K, d=150, m=m, lr=0.02)
+    worst, _ = run_and_compare(libpgc, w, 5, mode=mode)
+    assert worst < TOL                               # relative to the decode's own scale, sum |alpha| max |store|
