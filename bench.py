@@ -117,7 +117,7 @@ def roofline_model(w: W.Workload, peaks: dict):
     return "hbm", float(rows * grad_bytes_per_row(w)), "GB/s", peaks.get("hbm_gbs") or 6800.0
 
 
-def kernel_label(w: W.Workload, single: bool, dom: int) -> str:
+def kernel_label(w: W.Workload, single: bool, dom: int, split: bool) -> str:
     if tensor_core_path(w):
         nt = -(-w.K // 256)
         if dom == 2:
@@ -130,7 +130,7 @@ def kernel_label(w: W.Workload, single: bool, dom: int) -> str:
             return "softmax_rows_kernel (16-row tiles split by features over CTA pairs, one pass over X; whole step)"
         return "softmax_smallk_kernel (8-CTA clusters, one pass over X)"
     if w.loss == "softmax":
-        return "split_gemm_kernel (tcgen05, operands in bf16 parts)" if w.K <= 128 else "CUDA-core softmax gradient kernels"
+        return "split_gemm_kernel (tcgen05, operands in bf16 parts)" if split else "CUDA-core softmax gradient kernels"
     return "grad_rows kernel with fused commit+decode (whole step)" if single else "grad_rows kernel"
 
 
@@ -475,6 +475,7 @@ def measure(w: W.Workload, K_steps: int, Wu: int, seed: int, mode: str, cpu_seco
     peaks, peak_src = load_peaks()
     bound, units, unit, peak = roofline_model(w, peaks)
     single = all(n == 0 for n in tim["launches"][1:]) and tim["launches"][0] == tim["steps"]
+    split = tim["launches"][0] == 2 * tim["steps"]       # logits and gradient (the CUDA-core form launches three)
     dom = 0
     if tensor_core_path(w) and group_ms[2] > group_ms[0]:
         dom = 2
@@ -482,7 +483,7 @@ def measure(w: W.Workload, K_steps: int, Wu: int, seed: int, mode: str, cpu_seco
     scale = 1e9 if unit == "GB/s" else 1e12
     achieved = units / (grad_ms * 1e-3) / scale
     roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit, "frac": achieved / peak,
-                "peak_source": peak_src, "kernel": kernel_label(w, single, dom), "duration_ms": grad_ms,
+                "peak_source": peak_src, "kernel": kernel_label(w, single, dom, split), "duration_ms": grad_ms,
                 "traffic": recorded_traffic(w.name), "algorithmic_per_launch": units}
     if tensor_core_path(w):
         # the whole step against the burst rate: both contractions' flops

@@ -150,7 +150,7 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
   return __uint_as_float(static_cast<uint32_t>(b) << 16);
 }
 
-// Element loaders from a 16/8/4-byte vector held in registers.
+// Element loaders from a 16-byte vector held in registers.
 template <typename T, int VEC>
 struct Vec;
 
@@ -162,16 +162,6 @@ struct Vec<float, 4> {
   }
 };
 template <>
-struct Vec<float, 2> {
-  using raw = float2;
-  __device__ __forceinline__ static void widen(const raw& r, float* o) { o[0] = r.x; o[1] = r.y; }
-};
-template <>
-struct Vec<float, 1> {
-  using raw = float;
-  __device__ __forceinline__ static void widen(const raw& r, float* o) { o[0] = r; }
-};
-template <>
 struct Vec<uint16_t, 8> {
   using raw = uint4;
   __device__ __forceinline__ static void widen(const raw& r, float* o) {
@@ -181,21 +171,6 @@ struct Vec<uint16_t, 8> {
       o[2 * i] = __uint_as_float(w[i] << 16);
       o[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
     }
-  }
-};
-template <>
-struct Vec<uint16_t, 4> {
-  using raw = uint2;
-  __device__ __forceinline__ static void widen(const raw& r, float* o) {
-    o[0] = __uint_as_float(r.x << 16); o[1] = __uint_as_float(r.x & 0xffff0000u);
-    o[2] = __uint_as_float(r.y << 16); o[3] = __uint_as_float(r.y & 0xffff0000u);
-  }
-};
-template <>
-struct Vec<uint16_t, 2> {
-  using raw = uint32_t;
-  __device__ __forceinline__ static void widen(const raw& r, float* o) {
-    o[0] = __uint_as_float(r << 16); o[1] = __uint_as_float(r & 0xffff0000u);
   }
 };
 

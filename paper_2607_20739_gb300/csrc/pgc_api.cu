@@ -160,7 +160,7 @@ struct pgc_ctx {
   alignas(64) unsigned char tmXq[128];   // X as the fused kernel's A part (box 64 x 128/NT)
   alignas(64) unsigned char tmRst[128];  // Rb as the fused kernel's output (box 64 x 32)
   bool split = false;        // softmax in single precision on the tensor cores
-  int sp_nc = 0;             // its clusters of two CTAs
+  int sp_nc = 0;             // its clusters (of split_cluster CTAs)
   int sp_Kp = 0, sp_C3 = 0;  // classes padded to 16, columns of R
   int sp_h = kSplitTile;     // rows per CTA and logits unit
   uint16_t* R3 = nullptr;    // residual parts [R rows][C3]

@@ -415,7 +415,7 @@ struct SplitArgs {
   float2* row_stats;        // [ncb][rows]
   float* row_lab;           // [rows]
 };
-// Clusters of two CTAs that fit at once (0: cannot launch).
+// Clusters (of split_cluster CTAs) that fit at once (0: cannot launch).
 int split_max_clusters(int mode, int dtype, int64_t K);
 // kSplitLogits: R from X and W; tmB = W parts [3 Kp][ld], box {64, 3 Kp / cl}; tmX: box
 // {128 bytes, h} per partition, 128-byte swizzle.  kSplitGrad: partials (or stores) from R and X;

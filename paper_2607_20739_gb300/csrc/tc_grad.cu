@@ -10,7 +10,8 @@
 // CTAs owns the 256 x 256 output tile (class tiles 2mp, 2mp+1; feature tile
 // nt) for a run of up to eight partitions and computes G_e of each in turn.
 // Each CTA loads its 128 x 64 R tile and one half of the 64 x 256 X tile,
-// multicast into both CTAs, into a 4-stage ring (2-D TMA, 128-byte swizzle);
+// multicast into both CTAs, into a ring of stages (2-D TMA, 128-byte swizzle; four,
+// six in the pair form below, which is the default);
 // warp 1 issues tcgen05.mma (M = 128 classes, N = 256 features, K = 16 rows)
 // into one of two TMEM accumulators.  Eight epilogue warps (two per TMEM lane
 // quarter, 128 columns each) drain the other, 32 x 32 blocks at a time: a
