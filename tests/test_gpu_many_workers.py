@@ -43,3 +43,16 @@ def test_more_partitions_than_sms(libpgc, cuda, mode, scheme, n, s, dtype, d, m)
         assert rel_err(a["beta"], b["beta"]) < TOL
     assert all((g.store(i, 0) != 0).any() for i in range(n))
     g.close()
+
+
+@pytest.mark.parametrize("per_sm", ["1", "3"])
+@pytest.mark.parametrize("n,s,dtype,d,m", [(200, 1, "f32", 4096, 7), (3, 1, "f32", 600, (2049, 33, 1024)), (5, 1, "bf16", 1000, 700)])
+def test_items_handed_out_dynamically(libpgc, cuda, monkeypatch, per_sm, n, s, dtype, d, m):
+    """PGC_ITEMS_PER_SM: the CTAs take items of one length as they get free."""
+    monkeypatch.setenv("PGC_ITEMS_PER_SM", per_sm)
+    w = BASE.replace(n=n, s=s, dtype=dtype, d=d, m=m)
+    Xs, ys, masks = generate(w, 4)
+    g, recs = run_gpu(libpgc, w, Xs, ys, masks)
+    for a, b in zip(recs, run_oracle(w, Xs, ys, masks)):
+        assert rel_err(a["grad"], b["grad"]) < TOL
+    g.close()
