@@ -37,6 +37,11 @@
 //   now      63   62   62   62   62   61   62   67   67   63   71   72   76   86   86   67    72    73    76
 //   bf16    376  278  213  138  168   98   86  275  209  154  226  195  145  186  160  118   185   162   122
 //   now      64   77   64   66   80   62   61   86   75   68   84   81   75   90   84   71    95    90    98
+// Beyond 16384 bf16 features a lane's 160 to 256 columns of w and sums no longer fit
+// its registers (412 to 1296 bytes of spills per thread); still faster than before:
+//   d     16392 18000 20000 22528 24576 28000 32768
+//   bf16    442   414   378   344   320   289   252
+//   now     168   213   196   237   215   228   243
 // Item ends: consumers hand their accumulators to a tail warp (through a
 // shared buffer and two mbarriers) and keep streaming.  The tail warp sums the
 // teams' accumulators in a fixed order into the item's partial slot and,

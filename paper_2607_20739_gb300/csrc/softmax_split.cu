@@ -25,7 +25,10 @@
 //
 // Measured, us per step, before (three CUDA-core kernels) and with this file:
 // 12 partitions of 4096 x 3072 bf16, 100 classes: 3561 -> 222; 8 of 4096 x 784
-// fp32, 10 classes: 915 -> 60.  X is read once per kernel (twice per step).  The
+// fp32, 10 classes: 915 -> 60.  fp32 with 97 to 128 classes spills registers in the
+// epilogue's sums (logits 456 bytes per thread, gradient 324) and gains less: 12 of 4096 x 3072
+// 3540 -> 438 (97 classes) to 454 (128), 390 with 96; 4 of 300 x 700 131 -> 47 to 54.
+// X is read once per kernel (twice per step).  The
 // instructions of the single-thread roles bound an earlier form (282 and 102,
 // with ring positions divided out and descriptors rebuilt for every MMA).
 //
